@@ -99,11 +99,16 @@ typedef struct pr_opts {
     double aug_tol;         /* no augmentation if ||d~|| <= aug_tol ||U||; default 1e-12  */
     int group_ctas;         /* CTAs cooperating on one subinterval in the fine sweep (its
                                tile-planes split evenly over them; capped at their count);
-                               0: every co-resident CTA slot over the subintervals        */
+                               0: every co-resident CTA slot over the subintervals.
+                               Small grids (n <= 48 FP32, 34 FP64) run in the shared memory of
+                               one thread-block cluster a subinterval: 0 chooses its size, a
+                               positive value sets it (at most 16; n <= 40 FP32, 28 FP64)    */
     int ctas_per_sm;        /* resident CTAs per SM for the fine sweep; 0: occupancy max  */
     long long spin_limit;   /* polls of an in-kernel barrier or mbarrier before
                                PR_ERR_TIMEOUT (default 1<<22, a few seconds; 0: one
-                               non-blocking check, so a wait not already complete fails) */
+                               non-blocking check, so a wait not already complete fails).
+                               Clusters meet at a hardware barrier that polls nothing; with
+                               0 small grids keep the polling kernel                      */
     int method;             /* enum pr_method; default PR_METHOD_ADAPTIVE                 */
     int fine;               /* enum pr_fine; default PR_FINE_IMPLICIT_EULER               */
     int wave;               /* adaptive method only.  0 (default): pr_fine_sweep covers all

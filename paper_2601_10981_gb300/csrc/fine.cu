@@ -374,6 +374,12 @@ cudaError_t launch_fine(FineArgs a, bool fp32, int ctas_per_sm, int max_groups, 
     if (pt && (rk || td)) return cudaErrorInvalidValue;
     const int mode = rk ? FINE_MODE_RK4
                         : (td ? FINE_MODE_IMPLICIT_TD : (pt ? FINE_MODE_IMPLICIT_PERT : FINE_MODE_IMPLICIT));
+    // small grids: the on-chip kernel.  It has no wait that a spin limit could end, so a
+    // context that wants its waits to fail at once (spin_limit 0) keeps the polling kernel.
+    if ((mode == FINE_MODE_IMPLICIT || mode == FINE_MODE_IMPLICIT_PERT) && a.spin_limit > 0) {
+        ChipChoice ch;
+        if (fine_chip_plan(n, fp32, a.B, a.G, &ch)) return launch_fine_chip(a, fp32, ch, max_groups, st);
+    }
     FineFn fn = fine_select(n, fp32, mode);
     if (!fn) return cudaErrorInvalidValue;
     if (mode != FINE_MODE_IMPLICIT) {   // fine_max_ctas configured the steady instantiation

@@ -1409,4 +1409,14 @@ FineFn fine_fn_f32(int W, int KF, int KS, int mode);
 FineFn fine_fn_f64(int W, int KF, int KS, int mode);
 FineFn fine_fn_pert(bool fp32, int W, int KF, int KS);   // FINE_MODE_IMPLICIT_PERT (fine_pert.cu)
 
+// The same propagator on chip (fine_chip.cu): grids whose Krylov vectors fit the shared memory
+// of a cluster of C <= 16 CTAs (n <= 48 in the FP32 mode, 34 in FP64).  fine_chip_plan says
+// whether B subintervals run there, and how.
+struct ChipChoice {
+    int C, keep;
+    size_t smem;
+};
+bool fine_chip_plan(int n, bool fp32, int B, int group_ctas, ChipChoice* out);
+cudaError_t launch_fine_chip(const FineArgs& a, bool fp32, const ChipChoice& ch, int max_groups, cudaStream_t st);
+
 }  // namespace pr
