@@ -116,6 +116,7 @@ struct pr_ctx {
     double* ustc = nullptr;
     double* fpartc = nullptr;
     unsigned* fbarc = nullptr;
+    int* fresumec = nullptr;
     int max_ctas_c = 1;
     double* xc = nullptr;
     double* yc = nullptr;
@@ -143,6 +144,7 @@ struct pr_ctx {
     double* ust = nullptr;
     double* fpart = nullptr;
     unsigned* fbar = nullptr;
+    int* fresume = nullptr;
     int* fstatus = nullptr;
     int* fits = nullptr;
     int* fitsmax = nullptr;
@@ -242,8 +244,9 @@ size_t plan(pr_ctx* c, char* base) {
         c->fc32 = b.take<float>(Ngc);
         c->fwsc = b.take<char>(std::max((size_t)FINE_NVEC * Ngc * kesz2, (size_t)FINE_NVEC * Ngc * sizeof(double)));
         c->ustc = b.take<double>((size_t)2 * Ngc);
-        c->fpartc = b.take<double>((size_t)8 * c->max_ctas_c);
-        c->fbarc = b.take<unsigned>(2);
+        c->fpartc = b.take<double>(fine_part_doubles(c->max_ctas_c));
+        c->fbarc = b.take<unsigned>(4);
+        c->fresumec = b.take<int>(1);
         c->xc = b.take<double>(Ngc);
         c->yc = b.take<double>(Ngc);
         c->trajc = b.take<double>((size_t)(N + 1) * Ngc);
@@ -271,8 +274,9 @@ size_t plan(pr_ctx* c, char* base) {
                             (size_t)FINE_NVEC * Ng * sizeof(double));
     c->fws = b.take<char>(c->fws_bytes);
     c->ust = b.take<double>((size_t)c->groups_max * 2 * Ng);
-    c->fpart = b.take<double>((size_t)8 * c->max_ctas);
-    c->fbar = b.take<unsigned>((size_t)2 * c->groups_max);
+    c->fpart = b.take<double>(fine_part_doubles(c->max_ctas));
+    c->fbar = b.take<unsigned>((size_t)4 * c->groups_max);
+    c->fresume = b.take<int>(N + 1);
     c->fstatus = b.take<int>(N + 1);
     c->fits = b.take<int>(N + 1);
     c->fitsmax = b.take<int>(N + 1);
@@ -596,6 +600,7 @@ pr_status run_fine(pr_ctx* c, const double* u_in, double* u_out, char* snap, int
     J.snap = snap;
     J.tol = force_fp64 ? std::min(c->lin_tol, 1e-14) : c->lin_tol;
     J.maxit = c->o.lin_maxit;
+    J.resume = c->fresume + stat_off;
     J.status = c->fstatus + stat_off;
     J.its_total = c->fits + stat_off;
     J.its_max = c->fitsmax + stat_off;
@@ -606,11 +611,12 @@ pr_status run_fine(pr_ctx* c, const double* u_in, double* u_out, char* snap, int
     a.ust = c->ust;
     a.part = c->fpart;
     a.bar = c->fbar;
+    a.bar_groups = c->groups_max;
     a.G = c->o.group_ctas;
     a.spin_limit = c->o.spin_limit;
     a.err = c->derr;
     int max_groups = force_fp64 && c->fp32 ? 1 : c->groups_max;
-    PR_CUDA(cudaMemsetAsync(c->fbar, 0, sizeof(unsigned) * 2 * c->groups_max, c->st));
+    PR_CUDA(cudaMemsetAsync(c->fbar, 0, sizeof(unsigned) * 4 * c->groups_max, c->st));
     PR_CUDA(launch_fine(a, f32, c->o.ctas_per_sm, max_groups, c->st));
     return PR_OK;
 }
@@ -648,6 +654,7 @@ pr_status run_coarse_grid(pr_ctx* c, const double* x_in, double* y_out, double* 
     J.snap = snap;
     J.tol = c->lin_tol;
     J.maxit = c->o.lin_maxit;
+    J.resume = c->fresumec;
     J.status = c->fstatus + c->N;
     J.its_total = c->fits + c->N;
     J.its_max = c->fitsmax + c->N;
@@ -658,10 +665,11 @@ pr_status run_coarse_grid(pr_ctx* c, const double* x_in, double* y_out, double* 
     a.ust = c->ustc;
     a.part = c->fpartc;
     a.bar = c->fbarc;
+    a.bar_groups = 1;
     a.G = 0;
     a.spin_limit = c->o.spin_limit;
     a.err = c->derr;
-    PR_CUDA(cudaMemsetAsync(c->fbarc, 0, sizeof(unsigned) * 2, c->st));
+    PR_CUDA(cudaMemsetAsync(c->fbarc, 0, sizeof(unsigned) * 4, c->st));
     PR_CUDA(launch_fine(a, c->fp32, c->o.ctas_per_sm, 1, c->st));
     return PR_OK;
 }
@@ -1271,6 +1279,7 @@ pr_status pr_fine_sweep_batch(pr_ctx* const* ctxs, const int* ks, int count) {
         J.snap = plain ? nullptr : c->snap + (size_t)(k - 1) * c->ns * Ng * c->esz;
         J.tol = c->lin_tol;
         J.maxit = c->o.lin_maxit;
+        J.resume = c->fresume + (k - 1);
         J.status = c->fstatus + (k - 1);
         J.its_total = c->fits + (k - 1);
         J.its_max = c->fitsmax + (k - 1);
@@ -1282,6 +1291,7 @@ pr_status pr_fine_sweep_batch(pr_ctx* const* ctxs, const int* ks, int count) {
     a.ust = owner->ust;
     a.part = owner->fpart;
     a.bar = owner->fbar;
+    a.bar_groups = owner->groups_max;
     a.G = owner->o.group_ctas;
     a.spin_limit = owner->o.spin_limit;
     a.err = owner->derr;
@@ -1295,7 +1305,7 @@ pr_status pr_fine_sweep_batch(pr_ctx* const* ctxs, const int* ks, int count) {
     }
     {
         pr_ctx* c = owner;
-        PR_CUDA(cudaMemsetAsync(c->fbar, 0, sizeof(unsigned) * 2 * c->groups_max, c->st));
+        PR_CUDA(cudaMemsetAsync(c->fbar, 0, sizeof(unsigned) * 4 * c->groups_max, c->st));
         PR_CUDA(launch_fine(a, c->fp32, c->o.ctas_per_sm, c->groups_max, c->st));
         PR_CUDA(cudaEventRecord(c->ev[7], c->st));
     }

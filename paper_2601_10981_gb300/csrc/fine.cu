@@ -358,28 +358,19 @@ int fine_max_ctas(int n, bool fp32, int ctas_per_sm) {
     return std::max(1, occ) * std::max(1, sms);
 }
 
-cudaError_t launch_fine(FineArgs a, bool fp32, int ctas_per_sm, int max_groups, cudaStream_t st) {
-    if (a.B <= 0) return cudaSuccess;
+static int device_sms() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return std::max(1, sms);
+}
+
+// Doubles of the group reductions' partials: two sets of up to five products a CTA.
+size_t fine_part_doubles(int max_ctas) { return (size_t)10 * std::max(max_ctas, 4 * device_sms()); }
+
+// fine_kernel in the instantiation for the grid and mode.
+static cudaError_t launch_streaming(FineArgs a, bool fp32, int mode, int ctas_per_sm, int max_groups, cudaStream_t st) {
     const int n = a.g.n;
-    if (n > 256 || n < 4) return cudaErrorInvalidValue;
-    const bool rk = a.jobs[0].rk4 != 0;
-    const bool pt = a.jobs[0].pert != nullptr;
-    bool td = false;
-    for (int j = 0; j < a.njobs; ++j) {
-        if ((a.jobs[j].rk4 != 0) != rk) return cudaErrorInvalidValue;   // one integrator per launch
-        if ((a.jobs[j].pert != nullptr) != pt) return cudaErrorInvalidValue;   // one stencil kind
-        td = td || a.jobs[j].tdep != 0;
-    }
-    // the perturbation is a steady field of the implicit propagator
-    if (pt && (rk || td)) return cudaErrorInvalidValue;
-    const int mode = rk ? FINE_MODE_RK4
-                        : (td ? FINE_MODE_IMPLICIT_TD : (pt ? FINE_MODE_IMPLICIT_PERT : FINE_MODE_IMPLICIT));
-    // small grids: the on-chip kernel.  It has no wait that a spin limit could end, so a
-    // context that wants its waits to fail at once (spin_limit 0) keeps the polling kernel.
-    if ((mode == FINE_MODE_IMPLICIT || mode == FINE_MODE_IMPLICIT_PERT) && a.spin_limit > 0) {
-        ChipChoice ch;
-        if (fine_chip_plan(n, fp32, a.B, a.G, &ch)) return launch_fine_chip(a, fp32, ch, max_groups, st);
-    }
     FineFn fn = fine_select(n, fp32, mode);
     if (!fn) return cudaErrorInvalidValue;
     if (mode != FINE_MODE_IMPLICIT) {   // fine_max_ctas configured the steady instantiation
@@ -406,6 +397,55 @@ cudaError_t launch_fine(FineArgs a, bool fp32, int ctas_per_sm, int max_groups, 
     cudaError_t e = cudaLaunchCooperativeKernel((const void*)fn, dim3(grid), dim3(geo.threads), args, geo.smem, st);
     ++g_launch_count;
     return e;
+}
+
+cudaError_t launch_fine(FineArgs a, bool fp32, int ctas_per_sm, int max_groups, cudaStream_t st) {
+    if (a.B <= 0) return cudaSuccess;
+    const int n = a.g.n;
+    if (n > 256 || n < 4) return cudaErrorInvalidValue;
+    const bool rk = a.jobs[0].rk4 != 0;
+    const bool pt = a.jobs[0].pert != nullptr;
+    bool td = false;
+    for (int j = 0; j < a.njobs; ++j) {
+        if ((a.jobs[j].rk4 != 0) != rk) return cudaErrorInvalidValue;   // one integrator per launch
+        if ((a.jobs[j].pert != nullptr) != pt) return cudaErrorInvalidValue;   // one stencil kind
+        td = td || a.jobs[j].tdep != 0;
+    }
+    // the perturbation is a steady field of the implicit propagator
+    if (pt && (rk || td)) return cudaErrorInvalidValue;
+    const int mode = rk ? FINE_MODE_RK4
+                        : (td ? FINE_MODE_IMPLICIT_TD : (pt ? FINE_MODE_IMPLICIT_PERT : FINE_MODE_IMPLICIT));
+    // small grids: the on-chip kernel.  It has no wait that a spin limit could end, so a
+    // context that wants its waits to fail at once (spin_limit 0) keeps the polling kernel.
+    if ((mode == FINE_MODE_IMPLICIT || mode == FINE_MODE_IMPLICIT_PERT) && a.spin_limit > 0) {
+        ChipChoice ch;
+        if (fine_chip_plan(n, fp32, a.B, a.G, &ch)) return launch_fine_chip(a, fp32, ch, max_groups, st);
+    }
+    // Large grids of the FP32 mode: fine_kernel for the first step, fused_kernel, and fine_kernel
+    // again for the items it leaves (usually none).  The group size is the caller's in each.
+    // The second launch reads both u_0 and u_1, which u_out holds: not in place.
+    bool in_place = false;
+    for (int j = 0; j < a.njobs; ++j) {
+        const FineJob& J = a.jobs[j];
+        const size_t len = (size_t)J.B * a.g.Ng;
+        in_place = in_place || (J.u_in < J.u_out + len && J.u_out < J.u_in + len);
+    }
+    if (mode == FINE_MODE_IMPLICIT && fp32 && a.spin_limit > 0 && !in_place && fine_fused_takes(n)) {
+        FineArgs first = a;
+        int most = 0;
+        for (int j = 0; j < a.njobs; ++j) {
+            most = std::max(most, a.jobs[j].S);
+            first.jobs[j].S = 1;
+            first.jobs[j].resume = nullptr;
+        }
+        cudaError_t e = launch_streaming(first, fp32, mode, ctas_per_sm, max_groups, st);
+        if (e != cudaSuccess || most == 1) return e;
+        e = launch_fine_fused(a, max_groups, st);
+        if (e != cudaSuccess) return e;
+        return launch_streaming(a, fp32, mode, ctas_per_sm, max_groups, st);
+    }
+    for (int j = 0; j < a.njobs; ++j) a.jobs[j].resume = nullptr;
+    return launch_streaming(a, fp32, mode, ctas_per_sm, max_groups, st);
 }
 
 } // namespace pr

@@ -90,55 +90,6 @@ __device__ __forceinline__ T* chip_peer(T* p, unsigned rank) {
     return reinterpret_cast<T*>(o);
 }
 
-// Warp sums of NQ values a lane, halving the values a lane holds while the lanes that share
-// one double (9 additions for 5 values where 5 separate trees take 25).  Afterwards the lanes
-// whose low bits are zero hold value `q` (returned; -1: none).
-template <typename T, int NQ>
-__device__ __forceinline__ int chip_warp_sums(T (&v)[NQ], T& out) {
-    const int lane = threadIdx.x & 31;
-    constexpr unsigned M = 0xffffffffu;
-    if constexpr (NQ == 1) {
-        T x = v[0];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(M, x, o);
-        out = x;
-        return lane == 0 ? 0 : -1;
-    } else if constexpr (NQ == 2) {
-        const bool up = lane & 16;
-        T x = (up ? v[1] : v[0]) + __shfl_xor_sync(M, up ? v[0] : v[1], 16);
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(M, x, o);
-        out = x;
-        return (lane & 15) == 0 ? (lane >> 4) : -1;
-    } else if constexpr (NQ == 4) {
-        const bool u16 = lane & 16, u8 = lane & 8;
-        const T w0 = (u16 ? v[2] : v[0]) + __shfl_xor_sync(M, u16 ? v[0] : v[2], 16);
-        const T w1 = (u16 ? v[3] : v[1]) + __shfl_xor_sync(M, u16 ? v[1] : v[3], 16);
-        T z = (u8 ? w1 : w0) + __shfl_xor_sync(M, u8 ? w0 : w1, 8);
-#pragma unroll
-        for (int o = 4; o > 0; o >>= 1) z += __shfl_xor_sync(M, z, o);
-        out = z;
-        return (lane & 7) == 0 ? (u16 ? 2 : 0) + (u8 ? 1 : 0) : -1;
-    } else {
-        static_assert(NQ == 5, "1, 2, 4 or 5 values");
-        const bool u16 = lane & 16, u8 = lane & 8, u4 = lane & 4;
-        // value 4 goes to the upper half, paired with 0; 1..3 are added in the lower half only
-        T w0 = (u16 ? v[4] : v[0]) + __shfl_xor_sync(M, u16 ? v[0] : v[4], 16);
-        T w1 = v[1] + __shfl_xor_sync(M, v[1], 16);
-        T w2 = v[2] + __shfl_xor_sync(M, v[2], 16);
-        T w3 = v[3] + __shfl_xor_sync(M, v[3], 16);
-        T y0 = (u8 ? w2 : w0) + __shfl_xor_sync(M, u8 ? w0 : w2, 8);
-        T y1 = (u8 ? w3 : w1) + __shfl_xor_sync(M, u8 ? w1 : w3, 8);
-        T z = (u4 ? y1 : y0) + __shfl_xor_sync(M, u4 ? y0 : y1, 4);
-        z += __shfl_xor_sync(M, z, 2);
-        z += __shfl_xor_sync(M, z, 1);
-        out = z;
-        if (lane & 3) return -1;
-        const int q = (u8 ? 2 : 0) + (u4 ? 1 : 0);
-        return u16 ? (q == 0 ? 4 : -1) : q;
-    }
-}
-
 template <typename KT, int W, bool PT>
 __global__ void __launch_bounds__(512, 1) fine_chip_kernel(FineArgs a, ChipPlan cp) {
     constexpr bool DF = std::is_same<KT, float>::value;   // double-float state
@@ -342,21 +293,23 @@ __global__ void __launch_bounds__(512, 1) fine_chip_kernel(FineArgs a, ChipPlan 
                 kp = (KT)sc;
             }
             const double* tb = J.tab;
-            auto put = [&](KT* up, KT* dn, int i, double vel) {
-                if constexpr (DF) up[i] = (KT)(vel * sc);
-                else {
-                    up[i] = vel * sc - d1;
-                    dn[i] = -(vel * sc + d1);
+            // velocity va + vb.  FP32: each part scaled and rounded by itself, as fine_kernel does
+            auto put = [&](KT* up, KT* dn, int i, double va, double vb) {
+                if constexpr (DF) {
+                    up[i] = (KT)(va * J.dt * 0.5 / h) + (KT)(vb * J.dt * 0.5 / h);
+                } else {
+                    up[i] = (va + vb) * sc - d1;
+                    dn[i] = -((va + vb) * sc + d1);
                 }
             };
             for (int i = tid; i < npl * n; i += nthr) {
                 const int z = i / n, k = i - z * n;
-                put(ax, bx, i, tb[TXY * n + k] + tb[TXZ * n + z0 + z]);
-                put(ay, by, i, tb[TYX * n + k] + tb[TYZ * n + z0 + z]);
+                put(ax, bx, i, tb[TXY * n + k], tb[TXZ * n + z0 + z]);
+                put(ay, by, i, tb[TYX * n + k], tb[TYZ * n + z0 + z]);
             }
             for (int i = tid; i < n2; i += nthr) {
                 const int y = i / n, x = i - y * n;
-                put(az, bz, i, tb[TZX * n + x] + tb[TZY * n + y]);
+                put(az, bz, i, tb[TZX * n + x], tb[TZY * n + y]);
             }
         }
         const int S = J.S, dM = J.dM, n_snap = J.n_snap;
@@ -791,17 +744,18 @@ static int chip_clusters(int C) {
 }
 
 // Whether a launch of B subintervals runs on chip, and in clusters of how many CTAs: the C of
-// the least estimated time a step, if that is below fine_kernel's.  The estimates (SM cycles)
-// are fits to measured launches: a part for the barriers, reductions and scalars, and one for
-// the points of a CTA's slab.  Against fine_kernel, 40 steps, ms: FP64 16^3 x 8 3.9 -> 1.24,
-// 24^3 x 32 11.0 -> 4.2, 28^3 x 64 22.8 -> 14.3, but 32^3 x 64 25.0 -> 28.3 (three planes a CTA
-// at most fit, so 11-CTA clusters in eight turns); FP32 16^3 x 16 1.27 -> 0.37, 32^3 x 64
-// 2.5 -> 1.5, 45^3 x 16 3.4 -> 2.5, but 44^3 x 64 5.8 -> 6.2.
+// the least estimated time a step, if that is below the streaming kernels'.  The estimates (SM
+// cycles) are fits to measured launches: a part for the barriers, reductions and scalars, and
+// one for the points of a CTA's slab.  Against them, 40 steps, ms: FP64 (fine_kernel) 16^3 x 8
+// 3.9 -> 1.24, 24^3 x 32 11.0 -> 4.2, 28^3 x 64 22.8 -> 14.3, but 32^3 x 64 25.0 -> 28.3 (three
+// planes a CTA at most fit, so 11-CTA clusters in eight turns); FP32 16^3 x 16 1.27 -> 0.37
+// (fine_kernel), 32^3 x 64 2.4 -> 1.5, 40^3 x 8 1.23 -> 0.75, but 40^3 x 64 2.8 -> 3.4 and
+// 48^3 x 16 2.0 -> 2.3 (fused_kernel), 45^3 x 16 3.4 -> 2.5 (fine_kernel).
 // A caller who fixes group_ctas gets that C (the nearest that fits) on the grids where the
 // cluster always wins, whatever B, and fine_kernel beyond: the result of a subinterval then
 // does not depend on how many share the launch.
 bool fine_chip_plan(int n, bool fp32, int B, int group_ctas, ChipChoice* out) {
-    if (n < 4 || (group_ctas > 0 && n > (fp32 ? 40 : 28))) return false;
+    if (n < 4 || (group_ctas > 0 && n > (fp32 ? 36 : 28))) return false;
     double best = 0.0;
     out->C = 0;
     const double n2 = (double)n * n;
@@ -832,7 +786,8 @@ bool fine_chip_plan(int n, bool fp32, int B, int group_ctas, ChipChoice* out) {
     if (out->C == 0) return false;
     if (group_ctas > 0) return true;
     const double pts = B * n2 * n;
-    const double streamed = fp32 ? 45000.0 + (n % 4 ? 0.11 : 0.048) * pts : 150000.0 + (n % 4 ? 0.95 : 0.55) * pts;
+    const double streamed = fp32 ? (n % 4 ? 45000.0 + 0.11 * pts : 50000.0 + 0.023 * pts)
+                                 : 150000.0 + (n % 4 ? 0.95 : 0.55) * pts;
     return best < streamed;
 }
 

@@ -127,9 +127,58 @@ __device__ __forceinline__ void cta_sum(Acc<KT, NQ>& acc, double* red) {
     }
 }
 
+// Warp sums of NQ values a lane, halving the values a lane holds while the lanes that share
+// one double (9 additions for 5 values where 5 separate trees take 25).  Afterwards the lanes
+// whose low bits are zero hold value `q` (returned; -1: none).
+template <typename T, int NQ>
+__device__ __forceinline__ int chip_warp_sums(T (&v)[NQ], T& out) {
+    const int lane = threadIdx.x & 31;
+    constexpr unsigned M = 0xffffffffu;
+    if constexpr (NQ == 1) {
+        T x = v[0];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(M, x, o);
+        out = x;
+        return lane == 0 ? 0 : -1;
+    } else if constexpr (NQ == 2) {
+        const bool up = lane & 16;
+        T x = (up ? v[1] : v[0]) + __shfl_xor_sync(M, up ? v[0] : v[1], 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(M, x, o);
+        out = x;
+        return (lane & 15) == 0 ? (lane >> 4) : -1;
+    } else if constexpr (NQ == 4) {
+        const bool u16 = lane & 16, u8 = lane & 8;
+        const T w0 = (u16 ? v[2] : v[0]) + __shfl_xor_sync(M, u16 ? v[0] : v[2], 16);
+        const T w1 = (u16 ? v[3] : v[1]) + __shfl_xor_sync(M, u16 ? v[1] : v[3], 16);
+        T z = (u8 ? w1 : w0) + __shfl_xor_sync(M, u8 ? w0 : w1, 8);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) z += __shfl_xor_sync(M, z, o);
+        out = z;
+        return (lane & 7) == 0 ? (u16 ? 2 : 0) + (u8 ? 1 : 0) : -1;
+    } else {
+        static_assert(NQ == 5, "1, 2, 4 or 5 values");
+        const bool u16 = lane & 16, u8 = lane & 8, u4 = lane & 4;
+        // value 4 goes to the upper half, paired with 0; 1..3 are added in the lower half only
+        T w0 = (u16 ? v[4] : v[0]) + __shfl_xor_sync(M, u16 ? v[0] : v[4], 16);
+        T w1 = v[1] + __shfl_xor_sync(M, v[1], 16);
+        T w2 = v[2] + __shfl_xor_sync(M, v[2], 16);
+        T w3 = v[3] + __shfl_xor_sync(M, v[3], 16);
+        T y0 = (u8 ? w2 : w0) + __shfl_xor_sync(M, u8 ? w0 : w2, 8);
+        T y1 = (u8 ? w3 : w1) + __shfl_xor_sync(M, u8 ? w1 : w3, 8);
+        T z = (u4 ? y1 : y0) + __shfl_xor_sync(M, u4 ? y0 : y1, 4);
+        z += __shfl_xor_sync(M, z, 2);
+        z += __shfl_xor_sync(M, z, 1);
+        out = z;
+        if (lane & 3) return -1;
+        const int q = (u8 ? 2 : 0) + (u4 ? 1 : 0);
+        return u16 ? (q == 0 ? 4 : -1) : q;
+    }
+}
+
 struct FineShared {
-    double red[4 * 32];
-    double sums[4];
+    double red[5 * 32];
+    double sums[8];
     // BiCGStab scalars and decisions, written by thread 0 after each group reduction:
     // GB300 runs FP64 divisions and square roots on its narrow FP64 pipe, so they are
     // taken once per CTA instead of once per thread
@@ -349,6 +398,7 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
     KT* Wk = reinterpret_cast<KT*>(a.ws) + (size_t)g * FINE_NVEC * Ng;
     KT* delta = Wk;
     KT* r = Wk + Ng;
+    KT* const rw = r;
     KT* rh = Wk + 2 * Ng;
     KT* p0 = Wk + 3 * Ng;
     KT* p1 = Wk + 4 * Ng;
@@ -421,212 +471,21 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
             kz_x[e] = tabk[TZX * n + x0 + e];
         }
     };
-    KT kx_y[KS], kz_y[KS];
-    KT kx_z = 0, ky_z = 0;
-    auto tile_terms = [&](int y0) {
-#pragma unroll
-        for (int k = 0; k < KS; ++k) {
-            const int y = min(y0 + ty + k * RP, n - 1);
-            kx_y[k] = tabk[TXY * n + y];
-            kz_y[k] = tabk[TZY * n + y];
+#include "fine_march.inl"
+    // Sums of a phase's dot products over the group, then post(sums) in thread 0, and the
+    // barrier between phases; false: the barrier gave up.
+    auto finish = [&](auto& acc, auto&& post) -> bool {
+        constexpr int NQ = sizeof(acc.s) / sizeof(KT);
+        acc.flush();
+        cta_sum<KT, NQ>(acc, sh.red);
+        if (threadIdx.x == 0) {
+            for (int qq = 0; qq < NQ; ++qq) part[(size_t)((ph & 1) * 4 + qq) * grid + blockIdx.x] = acc.d[qq];
         }
+        if (!group_barrier(bar, G, a.spin_limit, a.err)) return false;
+        group_sums(part + (size_t)(ph & 1) * 4 * grid, grid, g0, G, NQ, sh.sums, post);
+        ++ph;
+        return true;
     };
-    auto plane_terms = [&](int z) {
-        kx_z = tabk[TXZ * n + z];
-        ky_z = tabk[TYZ * n + z];
-    };
-
-    // The x +- 1 neighbours of the W points: shifts of the centre vector plus one edge
-    // value on each side read from the ring row.
-    auto shift = [&](const auto* row, const auto& c, auto& xp, auto& xm) {
-#pragma unroll
-        for (int e = 0; e < W - 1; ++e) {
-            xp.v[e] = c.v[e + 1];
-            xm.v[e + 1] = c.v[e];
-        }
-        xp.v[W - 1] = row[xr];
-        xm.v[0] = row[xl];
-    };
-
-    // ---- tile march for stencil phases (ring of FINE_SLOTS planes, one barrier per
-    // FINE_PLANES planes):
-    //   load(i) -> Raw            inputs of the operand at the W points from index i
-    //   opnd(Raw) -> Vec          operand values written into the ring
-    //   own(i) -> Own             inputs the output needs at owned points
-    //   out(i, k, y, Own, rowc, rowzp, rowzm)   per owned W points (k: row slot); rowc is
-    //                             the ring row of the points, rowzp / rowzm the rows above /
-    //                             below in z; rowc +- n are the y neighbours
-    // Plane p lives in slot (p - zlo + 1) mod FINE_SLOTS.  A round at z commits planes
-    // z+1 .. z+np (np <= PL), then the barrier, then the stencils of planes z .. z+np-1
-    // read planes z-1 .. z+np.  A thread that runs ahead can only reach the commits of
-    // the next round, planes z+np+1 .. z+2np, whose slots differ from those of z-1 .. z+np
-    // as long as 2 PL + 2 <= FINE_SLOTS; the next barrier stops it there.
-    //   pipe                       true: prefetch the next round's first plane during the
-    //                              stencils; false: load each plane just before committing
-    //                              it (fewer live registers)
-    auto march = [&](bool pipe, auto* ring, auto&& load, auto&& opnd, auto&& own, auto&& out) {
-        using Raw = decltype(load(0));
-        using Own = decltype(own(0));
-        constexpr int PL = FINE_PLANES, NSL = FINE_SLOTS;
-        for (int tt = t_lo; tt < t_hi; ++tt) {
-            int y0, zlo, zhi;
-            geo.tile(tt, y0, zlo, zhi);
-            tile_terms(y0);
-            int fidx[KF];
-#pragma unroll
-            for (int k = 0; k < KF; ++k) {
-                const int rr = ty + k * RP;
-                int y = y0 + rr - 1;
-                y = (y < 0) ? y + n : (y >= n ? y - n : y);
-                fidx[k] = (rr < RW) ? y * n + x0 : -1;   // in-plane offset, -1: no row
-            }
-            Raw pre[KF];
-            Own opre[KS];
-            auto prefetch = [&](int zp) {
-                const int zz = (zp < 0) ? zp + n : (zp >= n ? zp - n : zp);
-#pragma unroll
-                for (int k = 0; k < KF; ++k)
-                    if (fidx[k] >= 0) pre[k] = load(zz * n2 + fidx[k]);
-            };
-            auto own_of = [&](int z, Own (&dst)[KS]) {
-#pragma unroll
-                for (int k = 0; k < KS; ++k)
-                    if (ty + k * RP < TY) dst[k] = own(z * n2 + (y0 + ty + k * RP) * n + x0);
-            };
-            auto slot = [&](int p) { return (p - zlo + 1) % NSL; };
-            auto commit = [&](int sl) {
-#pragma unroll
-                for (int k = 0; k < KF; ++k) {
-                    const int rr = ty + k * RP;
-                    if (fidx[k] < 0) continue;
-                    auto* dst = ring + (sl * RW + rr) * n + x0;
-                    const auto val = opnd(pre[k]);
-                    if constexpr (is_hilo<std::decay_t<decltype(val)>>::value) {
-                        vstore(dst, val.hi);
-                        vstore(dst + ring_lo, val.lo);
-                    } else if constexpr (is_ophilo<std::decay_t<decltype(val)>>::value) {
-                        vstore(dst, val.op);
-                        vstore(dst + ring_lo, val.hi);
-                        vstore(dst + 2 * ring_lo, val.lo);
-                    } else {
-                        vstore(dst, val);
-                    }
-                }
-            };
-            prefetch(zlo - 1);
-            commit(0);
-            prefetch(zlo);
-            commit(1);
-            if (pipe) {
-                prefetch(zlo + 1);
-                own_of(zlo, opre);
-            }
-            for (int z = zlo; z < zhi; z += PL) {
-                const int np = min(PL, zhi - z);
-#pragma unroll
-                for (int q = 1; q <= PL; ++q) {
-                    if (q > np) break;
-                    if (!pipe || q > 1) prefetch(z + q);
-                    commit(slot(z + q));
-                }
-                __syncthreads();
-                Own cur[PL][KS];
-                if (pipe) {
-#pragma unroll
-                    for (int k = 0; k < KS; ++k) cur[0][k] = opre[k];
-#pragma unroll
-                    for (int q = 1; q < PL; ++q)
-                        if (q < np) own_of(z + q, cur[q]);
-                    if (z + np < zhi) {
-                        prefetch(z + np + 1);
-                        own_of(z + np, opre);
-                    }
-                } else {
-#pragma unroll
-                    for (int q = 0; q < PL; ++q)
-                        if (q < np) own_of(z + q, cur[q]);
-                }
-#pragma unroll
-                for (int q = 0; q < PL; ++q) {
-                    if (q >= np) break;
-                    const int zq = z + q;
-                    const int sc = slot(zq), sp = slot(zq + 1), sm = slot(zq - 1);
-                    plane_terms(zq);
-#pragma unroll
-                    for (int k = 0; k < KS; ++k) {
-                        const int rr = ty + k * RP;
-                        if (rr >= TY) continue;
-                        out(zq * n2 + (y0 + rr) * n + x0, k, y0 + rr, cur[q][k], ring + (sc * RW + rr + 1) * n,
-                            ring + (sp * RW + rr + 1) * n, ring + (sm * RW + rr + 1) * n);
-                    }
-                }
-            }
-            __syncthreads();   // the next tile's prologue rewrites slots 0 and 1
-        }
-    };
-    // ---- pointwise loop over owned points, one plane of KS rows at a time
-    auto owned = [&](auto&& load, auto&& fn) {
-        using Raw = decltype(load(0));
-        for (int tt = t_lo; tt < t_hi; ++tt) {
-            int y0, zlo, zhi;
-            geo.tile(tt, y0, zlo, zhi);
-            for (int z = zlo; z < zhi; ++z) {
-                Raw v[KS];
-#pragma unroll
-                for (int k = 0; k < KS; ++k)
-                    if (ty + k * RP < TY) v[k] = load(z * n2 + (y0 + ty + k * RP) * n + x0);
-#pragma unroll
-                for (int k = 0; k < KS; ++k)
-                    if (ty + k * RP < TY) fn(z * n2 + (y0 + ty + k * RP) * n + x0, v[k]);
-            }
-        }
-    };
-    // The 7-point operand values of the W points from ring rows (vector loads).
-    auto nb7 = [&](const auto* rowc, const auto* rowzp, const auto* rowzm) {
-        using T = std::remove_const_t<std::remove_pointer_t<decltype(rowc)>>;
-        Nb7<T, W> o;
-        o.c = vload<T, W>(rowc + x0);
-        shift(rowc, o.c, o.xp, o.xm);
-        o.yp = vload<T, W>(rowc + n + x0);
-        o.ym = vload<T, W>(rowc - n + x0);
-        o.zp = vload<T, W>(rowzp + x0);
-        o.zm = vload<T, W>(rowzm + x0);
-        return o;
-    };
-    // The stored perturbation at the W points from index i (FINE_MODE_IMPLICIT_PERT).  It is
-    // loaded where the stencil uses it, not one plane ahead with the other owned-point
-    // inputs: its 3 W registers held across the march made the instantiation spill.
-    auto load_pert = [&](int i) -> PertV<KT, W, PT> {
-        PertV<KT, W, PT> o;
-        if constexpr (PT) {
-            o.x = vload<KT, W>(bpk + i);
-            o.y = vload<KT, W>(bpk + Ng + i);
-            o.z = vload<KT, W>(bpk + 2 * Ng + i);
-        }
-        return o;
-    };
-    // A = I + dt L at the W points of row slot k (pb: the perturbation there)
-    auto applyA = [&](int k, const Vec<KT, W>& c, const Vec<KT, W>& xp, const Vec<KT, W>& xm,
-                      const Vec<KT, W>& yp, const Vec<KT, W>& ym, const Vec<KT, W>& zp,
-                      const Vec<KT, W>& zm, const PertV<KT, W, PT>& pb) -> Vec<KT, W> {
-        Vec<KT, W> o;
-#pragma unroll
-        for (int e = 0; e < W; ++e) {
-            KT ax = kx_y[k] + kx_z;
-            KT ay = ky_x[e] + ky_z;
-            KT az = kz_x[e] + kz_y[k];
-            if constexpr (PT) {
-                ax += kp * pb.x.v[e];
-                ay += kp * pb.y.v[e];
-                az += kp * pb.z.v[e];
-            }
-            o.v[e] = c0 * c.v[e] + (ax - c1) * xp.v[e] - (ax + c1) * xm.v[e] + (ay - c1) * yp.v[e] -
-                     (ay + c1) * ym.v[e] + (az - c1) * zp.v[e] - (az + c1) * zm.v[e];
-        }
-        return o;
-    };
-    using VK = Vec<KT, W>;
-    using VD = Vec<double, W>;
 
     for (int b = g; b < a.B; b += a.numGroups) {
         // job of item b and its index lb within the job
@@ -634,8 +493,11 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
         while (jb + 1 < a.njobs && lb >= a.jobs[jb].B) lb -= a.jobs[jb++].B;
         if (jb != cur_job) load_job(jb);
         const FineJob& J = a.jobs[jb];
+        // an item that fused_kernel left (J.resume): from its step j0 on, its state in u_out
+        const int j0 = J.resume ? J.resume[lb] : 1;
+        if (j0 == 0) continue;
         const int S = J.S, dM = J.dM, n_snap = J.n_snap;
-        const double* u_in = J.u_in + (size_t)lb * Ng;
+        const double* u_in = (J.resume ? J.u_out : J.u_in) + (size_t)lb * Ng;
         double* snap_b = J.snap ? reinterpret_cast<double*>(J.snap) + (size_t)lb * n_snap * Ng : nullptr;
         long long its_total = 0;
         int its_max = 0;
@@ -826,12 +688,12 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
                 }
             }
         } else {
-        for (int j = 1; j <= S; ++j) {
+        for (int j = j0; j <= S; ++j) {
             if (tdep) step_tables(J, t_item + j * dt);
             // ---------------- setup: u_{j-1} = u_{j-2} + delta ; r = rhat = dt (f - L u_{j-1})
-            const double* P = (j <= 2) ? u_in : ust + (size_t)((j - 2) & 1) * Ng;
-            double* Wt = (j >= 2) ? ust + (size_t)((j - 1) & 1) * Ng : nullptr;
-            const bool use_d = (j >= 2) && dvalid;
+            const double* P = (j <= j0 + 1) ? u_in : ust + (size_t)((j - 2) & 1) * Ng;
+            double* Wt = (j > j0) ? ust + (size_t)((j - 1) & 1) * Ng : nullptr;
+            const bool use_d = (j > j0) && dvalid;
             // FP32 mode: BiCGStab starts from the previous increment (the FP64 mode starts
             // from 0, i.e. from u_{j-1}, like the plain definition)
             const bool xg = DF && use_d;
@@ -903,7 +765,7 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
                       });
             } else {
                 // double-float state: the same residual, FP32 arithmetic only
-                const float2* Pf = (j <= 2) ? nullptr : reinterpret_cast<const float2*>(P);
+                const float2* Pf = (j <= j0 + 1) ? nullptr : reinterpret_cast<const float2*>(P);
                 float2* Wf = reinterpret_cast<float2*>(Wt);
                 const float* ff = J.f32;
                 const KT dtf = (KT)dt;
@@ -1012,16 +874,7 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
                           acc.tick();
                       });
             }
-            {
-                acc.flush();
-                cta_sum<KT, 2>(acc, sh.red);
-                if (threadIdx.x == 0) {
-                    part[(size_t)((ph & 1) * 4 + 0) * grid + blockIdx.x] = acc.d[0];
-                    part[(size_t)((ph & 1) * 4 + 1) * grid + blockIdx.x] = acc.d[1];
-                }
-            }
-            if (!group_barrier(bar, G, a.spin_limit, a.err)) return;
-            group_sums(part + (size_t)(ph & 1) * 4 * grid, grid, g0, G, 2, sh.sums, [&](const double* s) {
+            if (!finish(acc, [&](const double* s) {
                 const double rr0 = s[0], bb = s[1];
                 sh.thr = J.tol * sqrt(bb);
                 int conv = sqrt(rr0) <= sh.thr;
@@ -1031,262 +884,14 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
                 sh.alpha = 1.0;
                 sh.omega = 1.0;
                 sh.beta = 0.0;
-            });
-            ++ph;
+            })) return;
             const bool conv = sh.flag != 0;
             int it = 0;
-            while (!conv) {
-                ++it;
-                // ---------------- ph1: p = r + beta (p' - omega v'), v = A p
-                KT* pn = (it & 1) ? p1 : p0;
-                KT* po = (it & 1) ? p0 : p1;
-                KT* vn = (it & 1) ? v1 : v0;
-                KT* vo = (it & 1) ? v0 : v1;
-                {
-                    const KT bk = (KT)sh.beta, ok = (KT)sh.omega;
-                    const bool first = (it == 1);
-                    Acc<KT, 1> acc;
-                    acc.init();
-                    march(true, ringk,
-                          [&](int i) -> RawP<KT, W> {
-                              RawP<KT, W> o;
-                              o.r = vload<KT, W>(r + i);
-                              if (!first) {
-                                  o.p = vload<KT, W>(po + i);
-                                  o.v = vload<KT, W>(vo + i);
-                              } else {
-#pragma unroll
-                                  for (int e = 0; e < W; ++e) { o.p.v[e] = (KT)0; o.v.v[e] = (KT)0; }
-                              }
-                              return o;
-                          },
-                          [&](const RawP<KT, W>& v) -> VK {
-                              VK o;
-#pragma unroll
-                              for (int e = 0; e < W; ++e) o.v[e] = v.r.v[e] + bk * (v.p.v[e] - ok * v.v.v[e]);
-                              return o;
-                          },
-                          [&](int i) -> OwnH<KT, W, PT> { return {vload<KT, W>(rh + i), {}}; },
-                          [&](int i, int k, int, const OwnH<KT, W, PT>& ow, const KT* rowc, const KT* rowzp,
-                              const KT* rowzm) {
-                              const VK& rhv = ow.h;
-                              const auto q7 = nb7(rowc, rowzp, rowzm);
-                              const VK av = applyA(k, q7.c, q7.xp, q7.xm, q7.yp, q7.ym, q7.zp, q7.zm, load_pert(i));
-                              vstore(pn + i, q7.c);
-                              vstore(vn + i, av);
-#pragma unroll
-                              for (int e = 0; e < W; ++e) acc.f[0] += rhv.v[e] * av.v[e];
-                              acc.tick();
-                          });
-                    acc.flush();
-                    cta_sum<KT, 1>(acc, sh.red);
-                    if (threadIdx.x == 0) part[(size_t)((ph & 1) * 4) * grid + blockIdx.x] = acc.d[0];
-                }
-                if (!group_barrier(bar, G, a.spin_limit, a.err)) return;
-                group_sums(part + (size_t)(ph & 1) * 4 * grid, grid, g0, G, 1, sh.sums, [&](const double* s) {
-                    const double rv = s[0];
-                    if (rv == 0.0 || !isfinite(rv)) {
-                        sh.status = isfinite(rv) ? DERR_BREAKDOWN : DERR_NONFINITE;
-                        sh.flag = 1;
-                    } else {
-                        sh.alpha = sh.rho / rv;
-                        sh.flag = 0;
-                    }
-                });
-                ++ph;
-                if (sh.flag) {
-                    --it;
-                    break;
-                }
-                // ---------------- ph2: s = r - alpha v, t = A s
-                {
-                    const KT al = (KT)sh.alpha;
-                    Acc<KT, 3> acc;
-                    acc.init();
-                    march(true, ringk,
-                          [&](int i) -> RawS<KT, W> { return {vload<KT, W>(r + i), vload<KT, W>(vn + i)}; },
-                          [&](const RawS<KT, W>& v) -> VK {
-                              VK o;
-#pragma unroll
-                              for (int e = 0; e < W; ++e) o.v[e] = v.r.v[e] - al * v.v.v[e];
-                              return o;
-                          },
-                          [&](int) -> NoOwn { return NoOwn{}; },
-                          [&](int i, int k, int, const NoOwn&, const KT* rowc, const KT* rowzp,
-                              const KT* rowzm) {
-                              const auto q7 = nb7(rowc, rowzp, rowzm);
-                              const VK tv = applyA(k, q7.c, q7.xp, q7.xm, q7.yp, q7.ym, q7.zp, q7.zm, load_pert(i));
-                              vstore(t + i, tv);
-#pragma unroll
-                              for (int e = 0; e < W; ++e) {
-                                  acc.f[0] += tv.v[e] * q7.c.v[e];
-                                  acc.f[1] += tv.v[e] * tv.v[e];
-                                  acc.f[2] += q7.c.v[e] * q7.c.v[e];
-                              }
-                              acc.tick();
-                          });
-                    acc.flush();
-                    cta_sum<KT, 3>(acc, sh.red);
-                    if (threadIdx.x == 0) {
-                        for (int qq = 0; qq < 3; ++qq)
-                            part[(size_t)((ph & 1) * 4 + qq) * grid + blockIdx.x] = acc.d[qq];
-                    }
-                }
-                if (!group_barrier(bar, G, a.spin_limit, a.err)) return;
-                group_sums(part + (size_t)(ph & 1) * 4 * grid, grid, g0, G, 3, sh.sums, [&](const double* s) {
-                    const double ts = s[0], tt2 = s[1], ss = s[2];
-                    const int half = sqrt(ss) <= sh.thr;
-                    if (!half) {
-                        if (tt2 == 0.0 || !isfinite(tt2)) {
-                            sh.status = isfinite(tt2) ? DERR_BREAKDOWN : DERR_NONFINITE;
-                            sh.omega = 0.0;
-                        } else {
-                            sh.omega = ts / tt2;
-                            if (sh.omega == 0.0) sh.status = DERR_BREAKDOWN;
-                        }
-                    }
-                    sh.flag = half;
-                });
-                ++ph;
-                const bool half = sh.flag != 0;
-                // ---------------- ph3: delta += alpha p + omega s ; r = s - omega t
-                {
-                    const KT al = (KT)sh.alpha, om = (KT)sh.omega;
-                    const bool first = (it == 1) && !xg;   // delta holds the initial guess
-                    const bool upd_r = !half && sh.status == 0;
-                    Acc<KT, 2> acc;
-                    acc.init();
-                    // the update of the owned points from their six inputs
-                    auto p3_fn = [&](int i, const Raw6<KT, W>& v) {
-                        VK dn, rn;
-#pragma unroll
-                        for (int e = 0; e < W; ++e) {
-                            const KT sc_ = v.r.v[e] - al * v.v.v[e];
-                            dn.v[e] = v.d.v[e] + al * v.p.v[e] + om * sc_;
-                            rn.v[e] = sc_ - om * v.t.v[e];
-                            acc.f[0] += v.h.v[e] * rn.v[e];
-                            acc.f[1] += rn.v[e] * rn.v[e];
-                        }
-                        vstore(delta + i, dn);
-                        vstore(r + i, rn);
-                        acc.tick();
-                    };
-                    bool staged3 = false;
-                    if constexpr (DF && KS == 1) {
-                        if (upd_r) {
-                            // inputs of plane z staged by cp.async while planes z-2, z-1 are
-                            // updated; each thread reads back only what it copied, so no
-                            // barrier is needed; layout [slot][input][thread][W] (no bank
-                            // conflicts).  The ring is idle in this phase.
-                            staged3 = true;
-                            constexpr int NS = FINE_PH3_SLOTS;
-                            float* stg = reinterpret_cast<float*>(ring_raw);
-                            const int nthr = blockDim.x;
-                            const bool act = ty < TY;
-                            auto sad = [&](int sl, int q) { return stg + ((size_t)(sl * 6 + q) * nthr + threadIdx.x) * W; };
-                            for (int tt = t_lo; tt < t_hi; ++tt) {
-                                int y0, zlo, zhi;
-                                geo.tile(tt, y0, zlo, zhi);
-                                const int rowoff = (y0 + ty) * n + x0;
-                                auto issue = [&](int z, int sl) {
-                                    if (act && z < zhi) {
-                                        const long long i = (long long)z * n2 + rowoff;
-                                        if (!first) cp_async_b<4 * W>(sad(sl, 0), delta + i);
-                                        cp_async_b<4 * W>(sad(sl, 1), pn + i);
-                                        cp_async_b<4 * W>(sad(sl, 2), r + i);
-                                        cp_async_b<4 * W>(sad(sl, 3), vn + i);
-                                        cp_async_b<4 * W>(sad(sl, 4), t + i);
-                                        cp_async_b<4 * W>(sad(sl, 5), rh + i);
-                                    }
-                                    cp_async_commit_group();
-                                };
-#pragma unroll
-                                for (int d = 0; d < NS - 1; ++d) issue(zlo + d, d);
-                                int sl = 0;
-                                for (int z = zlo; z < zhi; ++z) {
-                                    // refill the slot of plane z - 1 (read last iteration)
-                                    issue(z + NS - 1, sl == 0 ? NS - 1 : sl - 1);
-                                    cp_async_wait_newest<NS - 1>();
-                                    if (act) {
-                                        Raw6<KT, W> v;
-                                        if (!first) v.d = vload<float, W>(sad(sl, 0));
-                                        else {
-#pragma unroll
-                                            for (int e = 0; e < W; ++e) v.d.v[e] = 0.0f;
-                                        }
-                                        v.p = vload<float, W>(sad(sl, 1));
-                                        v.r = vload<float, W>(sad(sl, 2));
-                                        v.v = vload<float, W>(sad(sl, 3));
-                                        v.t = vload<float, W>(sad(sl, 4));
-                                        v.h = vload<float, W>(sad(sl, 5));
-                                        p3_fn(z * n2 + rowoff, v);
-                                    }
-                                    sl = (sl + 1 == NS) ? 0 : sl + 1;
-                                }
-                                cp_async_wait_newest<0>();
-                            }
-                        }
-                    }
-                    if (upd_r && !staged3) {
-                        owned([&](int i) -> Raw6<KT, W> {
-                                  Raw6<KT, W> o;
-                                  if (!first) o.d = vload<KT, W>(delta + i);
-                                  else {
-#pragma unroll
-                                      for (int e = 0; e < W; ++e) o.d.v[e] = (KT)0;
-                                  }
-                                  o.p = vload<KT, W>(pn + i);
-                                  o.r = vload<KT, W>(r + i);
-                                  o.v = vload<KT, W>(vn + i);
-                                  o.t = vload<KT, W>(t + i);
-                                  o.h = vload<KT, W>(rh + i);
-                                  return o;
-                              },
-                              p3_fn);
-                    } else if (!upd_r) {
-                        owned([&](int i) -> RawP2<KT, W> {
-                                  RawP2<KT, W> o;
-                                  if (!first) o.d = vload<KT, W>(delta + i);
-                                  else {
-#pragma unroll
-                                      for (int e = 0; e < W; ++e) o.d.v[e] = (KT)0;
-                                  }
-                                  o.p = vload<KT, W>(pn + i);
-                                  return o;
-                              },
-                              [&](int i, const RawP2<KT, W>& v) {
-                                  VK dn;
-#pragma unroll
-                                  for (int e = 0; e < W; ++e) dn.v[e] = v.d.v[e] + al * v.p.v[e];
-                                  vstore(delta + i, dn);
-                              });
-                    }
-                    acc.flush();
-                    cta_sum<KT, 2>(acc, sh.red);
-                    if (threadIdx.x == 0 && upd_r) {
-                        part[(size_t)((ph & 1) * 4 + 0) * grid + blockIdx.x] = acc.d[0];
-                        part[(size_t)((ph & 1) * 4 + 1) * grid + blockIdx.x] = acc.d[1];
-                    }
-                    if (!group_barrier(bar, G, a.spin_limit, a.err)) return;
-                    if (!upd_r) break;
-                    group_sums(part + (size_t)(ph & 1) * 4 * grid, grid, g0, G, 2, sh.sums, [&](const double* s) {
-                        const double rho_new = s[0], rr1 = s[1];
-                        int stop = 1;
-                        if (!isfinite(rr1)) sh.status = DERR_NONFINITE;
-                        else if (sqrt(rr1) <= sh.thr) {}
-                        else if (rho_new == 0.0) sh.status = DERR_BREAKDOWN;
-                        else if (it >= J.maxit) sh.status = DERR_NOT_CONVERGED;
-                        else {
-                            sh.beta = (rho_new / sh.rho) * (sh.alpha / sh.omega);
-                            sh.rho = rho_new;
-                            stop = 0;
-                        }
-                        sh.flag = stop;
-                    });
-                    ++ph;
-                }
-                if (sh.flag) break;
-            }
+#define FINE_GIVE_UP
+#define FINE_PIPE true
+#include "fine_bicgstab.inl"
+#undef FINE_PIPE
+#undef FINE_GIVE_UP
             dvalid = it > 0 || xg;
             its_total += it;
             its_max = max(its_max, it);
@@ -1295,7 +900,7 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
         }
         // ---------------- final: u_S = u_{S-1} + delta ; snapshot of u_S
         {
-            const double* P = (S >= 2) ? ust + (size_t)((S - 1) & 1) * Ng : u_in;
+            const double* P = (S > j0) ? ust + (size_t)((S - 1) & 1) * Ng : u_in;
             double* snap_S = (snap_b && S % dM == 0 && S / dM < n_snap)
                                  ? snap_b + (size_t)(S / dM) * Ng : nullptr;
             double* outp = J.u_out + (size_t)lb * Ng;
@@ -1319,7 +924,7 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
                           if (snap_S) vstore(snap_S + i, u);
                       });
             } else {
-                const float2* Pf = (S >= 2) ? reinterpret_cast<const float2*>(P) : nullptr;
+                const float2* Pf = (S > j0) ? reinterpret_cast<const float2*>(P) : nullptr;
                 owned([&](int i) -> RawF<float2, KT, W> {
                           RawF<float2, KT, W> o;
                           if (Pf) o.u = vload<float2, W>(Pf + i);
@@ -1346,9 +951,9 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
         }
         }   // implicit Euler
         if (q == 0 && threadIdx.x == 0) {
-            J.status[lb] = sh.status;
-            J.its_total[lb] = (int)its_total;
-            J.its_max[lb] = its_max;
+            if (!J.resume || J.status[lb] == 0) J.status[lb] = sh.status;
+            J.its_total[lb] = (J.resume ? J.its_total[lb] : 0) + (int)its_total;
+            J.its_max[lb] = max(J.resume ? J.its_max[lb] : 0, its_max);
         }
         // The next subinterval's first setup reads only its own input state (and the
         // ring), and writes r/rhat at owned points, which no CTA of this group reads
@@ -1408,6 +1013,11 @@ using FineFn = void (*)(FineArgs);
 FineFn fine_fn_f32(int W, int KF, int KS, int mode);
 FineFn fine_fn_f64(int W, int KF, int KS, int mode);
 FineFn fine_fn_pert(bool fp32, int W, int KF, int KS);   // FINE_MODE_IMPLICIT_PERT (fine_pert.cu)
+
+// The FP32 mode's large grids in two passes a step (fine_fused.cu), steps 2 .. S after a launch of
+// the first one; whether the grid suits it.
+bool fine_fused_takes(int n);
+cudaError_t launch_fine_fused(FineArgs a, int max_groups, cudaStream_t st);
 
 // The same propagator on chip (fine_chip.cu): grids whose Krylov vectors fit the shared memory
 // of a cluster of C <= 16 CTAs (n <= 48 in the FP32 mode, 34 in FP64).  fine_chip_plan says

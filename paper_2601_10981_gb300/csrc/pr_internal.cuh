@@ -188,6 +188,8 @@ struct FineJob {
     int* its_total;     // [B]
     int* its_max;       // [B]
     int B;
+    int* resume;        // [B] the step at which fused_kernel left an item, 0: none; null: a launch
+                        // of fine_kernel that does all steps of all items
     const void* pert;   // stored velocity perturbation [3][Ng] in the Krylov type (float in
                         // the FP32 mode, double in FP64), unscaled, or nullptr
 };
@@ -200,11 +202,13 @@ struct FineArgs {
     int B;              // subintervals in this launch: the sum of jobs[].B
     void* ws;           // [numGroups][NVEC][Ng] of KT
     double* ust;        // [numGroups][2][Ng]
-    double* part;       // [numGroups][2][4][n]
-    unsigned* bar;      // [numGroups][2]
+    double* part;       // fine_part_doubles()
+    unsigned* bar;      // [2 bar_groups][2]: fine_kernel's groups, then fused_kernel's
+    int bar_groups;     // groups either half holds
     int G;              // CTAs per group
     int numGroups;
     int TY, NY;         // a subinterval: NY columns of TY rows, n tile-planes each
+    int fused_slots;    // fused_kernel: setup slots
     int RP;             // rows per pass of a CTA (threads = n/W lanes x RP, rounded to warps)
     long long spin_limit;
     int* err;           // launch-wide error code
@@ -217,6 +221,7 @@ cudaError_t launch_fine(FineArgs a, bool fp32, int ctas_per_sm, int max_groups,
                         cudaStream_t st);
 // Largest number of co-resident CTAs of the fine kernel for this grid size.
 int fine_max_ctas(int n, bool fp32, int ctas_per_sm);
+size_t fine_part_doubles(int max_ctas);   // FineArgs::part
 int fine_tile_rows(int n);
 int fine_block_threads(int n);
 
