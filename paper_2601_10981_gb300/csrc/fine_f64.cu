@@ -27,7 +27,7 @@ static FineFn pick_mode(int KF, int KS, int mode) {
 }
 
 FineFn fine_fn_f64(int W, int KF, int KS, int mode) {
-    return W == 4 ? pick_mode<4>(KF, KS, mode) : pick_mode<1>(KF, KS, mode);
+    return W == 2 ? pick_mode<2>(KF, KS, mode) : pick_mode<1>(KF, KS, mode);
 }
 
 }  // namespace pr

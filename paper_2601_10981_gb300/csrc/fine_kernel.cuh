@@ -238,6 +238,9 @@ __device__ __forceinline__ Vec<T, W> vload(const T* p) {
         const double2 q0 = *reinterpret_cast<const double2*>(p);
         const double2 q1 = *reinterpret_cast<const double2*>(p + 2);
         o.v[0] = q0.x; o.v[1] = q0.y; o.v[2] = q1.x; o.v[3] = q1.y;
+    } else if constexpr (W == 2 && sizeof(T) == 8) {
+        const double2 q0 = *reinterpret_cast<const double2*>(p);
+        o.v[0] = q0.x; o.v[1] = q0.y;
     } else {
 #pragma unroll
         for (int e = 0; e < W; ++e) o.v[e] = p[e];
@@ -254,6 +257,8 @@ __device__ __forceinline__ void vstore(T* p, const Vec<T, W>& o) {
     } else if constexpr (W == 4 && sizeof(T) == 8) {
         *reinterpret_cast<double2*>(p) = make_double2(o.v[0], o.v[1]);
         *reinterpret_cast<double2*>(p + 2) = make_double2(o.v[2], o.v[3]);
+    } else if constexpr (W == 2 && sizeof(T) == 8) {
+        *reinterpret_cast<double2*>(p) = make_double2(o.v[0], o.v[1]);
     } else {
 #pragma unroll
         for (int e = 0; e < W; ++e) p[e] = o.v[e];
@@ -383,6 +388,17 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
     constexpr bool DF = std::is_same<KT, float>::value;   // double-float state
     // float offset of the lo planes of the FP32-mode setup ring (the ring's upper half)
     const int ring_lo = FINE_SLOTS * (a.TY + 2) * n;
+    // FP64 implicit modes: weights of A = I + dt L at the neighbours in z ([+-][tile row][x]) and,
+    // for the plane at hand and the next, in y ([plane & 1][+-][x]).  GB300's FP64 pipe (2 FMAs
+    // a cycle and SM) bounds the FP64 mode, and forming the weights at each point took half of
+    // A's operations: A is now 7 FMAs a point, and <rhat, t> joins the products
+    // of the t phase, so the update phase needs none.  64^3, 16 subintervals x 32 steps: 68.0 ->
+    // 61.1 ms (the pipe 81 % busy); 96^3 x 8 x 10: 22.7 -> 18.0 ms; 128^3 x 8 x 10: 42.6 -> 38.1.
+    double* wz = ringd + (DF ? 0 : FINE_SLOTS * (a.TY + 2) * n);
+    double* wy = wz + 2 * a.TY * n;
+    constexpr bool WT = !DF && !RK;
+    (void)wz;
+    (void)wy;
     (void)ringd;
     // per-job constants (a launch can hold subintervals of several problems on the same
     // grid, see FineJob); set by load_job
@@ -398,7 +414,6 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
     KT* Wk = reinterpret_cast<KT*>(a.ws) + (size_t)g * FINE_NVEC * Ng;
     KT* delta = Wk;
     KT* r = Wk + Ng;
-    KT* const rw = r;
     KT* rh = Wk + 2 * Ng;
     KT* p0 = Wk + 3 * Ng;
     KT* p1 = Wk + 4 * Ng;
@@ -471,7 +486,267 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
             kz_x[e] = tabk[TZX * n + x0 + e];
         }
     };
-#include "fine_march.inl"
+    KT kx_y[KS], kz_y[KS];
+    KT kx_z = 0, ky_z = 0;
+    auto tile_terms = [&](int y0) {
+#pragma unroll
+        for (int k = 0; k < KS; ++k) {
+            const int y = min(y0 + ty + k * RP, n - 1);
+            kx_y[k] = tabk[TXY * n + y];
+            kz_y[k] = tabk[TZY * n + y];
+        }
+        if constexpr (WT) {   // read after the march's next barrier
+            for (int i = threadIdx.x; i < TY * n; i += blockDim.x) {
+                const int ry = i / n, x = i - ry * n;
+                const double az = tabk[TZX * n + x] + tabk[TZY * n + y0 + ry];
+                wz[i] = az - c1;
+                wz[TY * n + i] = -(az + c1);
+            }
+        }
+    };
+    int zcur = 0;   // the plane of the stencil
+    (void)zcur;
+    auto plane_terms = [&](int z) {
+        zcur = z;
+        kx_z = tabk[TXZ * n + z];
+        ky_z = tabk[TYZ * n + z];
+    };
+    // the y weights of plane z, by the first threads before the barrier that the stencil follows
+    auto plane_weights = [&](int z) {
+        if constexpr (WT) {
+            for (int x = threadIdx.x; x < n; x += blockDim.x) {
+                const double ay = tabk[TYX * n + x] + tabk[TYZ * n + z];
+                wy[(z & 1) * 2 * n + x] = ay - c1;
+                wy[(z & 1) * 2 * n + n + x] = -(ay + c1);
+            }
+        }
+    };
+
+    // The x +- 1 neighbours of the W points: shifts of the centre vector plus one edge
+    // value on each side read from the ring row.
+    auto shift = [&](const auto* row, const auto& c, auto& xp, auto& xm) {
+#pragma unroll
+        for (int e = 0; e < W - 1; ++e) {
+            xp.v[e] = c.v[e + 1];
+            xm.v[e + 1] = c.v[e];
+        }
+        xp.v[W - 1] = row[xr];
+        xm.v[0] = row[xl];
+    };
+
+    // ---- tile march for stencil phases (ring of FINE_SLOTS planes, one barrier per
+    // FINE_PLANES planes):
+    //   load(i) -> Raw            inputs of the operand at the W points from index i
+    //   opnd(Raw) -> Vec          operand values written into the ring
+    //   own(i) -> Own             inputs the output needs at owned points
+    //   out(i, k, y, Own, rowc, rowzp, rowzm)   per owned W points (k: row slot); rowc is
+    //                             the ring row of the points, rowzp / rowzm the rows above /
+    //                             below in z; rowc +- n are the y neighbours
+    // Plane p lives in slot (p - zlo + 1) mod FINE_SLOTS.  A round at z commits planes
+    // z+1 .. z+np (np <= PL), then the barrier, then the stencils of planes z .. z+np-1
+    // read planes z-1 .. z+np.  A thread that runs ahead can only reach the commits of
+    // the next round, planes z+np+1 .. z+2np, whose slots differ from those of z-1 .. z+np
+    // as long as 2 PL + 2 <= FINE_SLOTS; the next barrier stops it there.
+    //   pipe                       true: prefetch the next round's first plane during the
+    //                              stencils; false: load each plane just before committing
+    //                              it (fewer live registers)
+    auto march = [&](bool pipe, auto* ring, auto&& load, auto&& opnd, auto&& own, auto&& out) {
+        using Raw = decltype(load(0));
+        using Own = decltype(own(0));
+        constexpr int PL = FINE_PLANES, NSL = FINE_SLOTS;
+        for (int tt = t_lo; tt < t_hi; ++tt) {
+            int y0, zlo, zhi;
+            geo.tile(tt, y0, zlo, zhi);
+            tile_terms(y0);
+            int fidx[KF];
+#pragma unroll
+            for (int k = 0; k < KF; ++k) {
+                const int rr = ty + k * RP;
+                int y = y0 + rr - 1;
+                y = (y < 0) ? y + n : (y >= n ? y - n : y);
+                fidx[k] = (rr < RW) ? y * n + x0 : -1;   // in-plane offset, -1: no row
+            }
+            Raw pre[KF];
+            Own opre[KS];
+            auto prefetch = [&](int zp) {
+                const int zz = (zp < 0) ? zp + n : (zp >= n ? zp - n : zp);
+#pragma unroll
+                for (int k = 0; k < KF; ++k)
+                    if (fidx[k] >= 0) pre[k] = load(zz * n2 + fidx[k]);
+            };
+            auto own_of = [&](int z, Own (&dst)[KS]) {
+#pragma unroll
+                for (int k = 0; k < KS; ++k)
+                    if (ty + k * RP < TY) dst[k] = own(z * n2 + (y0 + ty + k * RP) * n + x0);
+            };
+            auto slot = [&](int p) { return (p - zlo + 1) % NSL; };
+            auto commit = [&](int sl) {
+#pragma unroll
+                for (int k = 0; k < KF; ++k) {
+                    const int rr = ty + k * RP;
+                    if (fidx[k] < 0) continue;
+                    auto* dst = ring + (sl * RW + rr) * n + x0;
+                    const auto val = opnd(pre[k]);
+                    if constexpr (is_hilo<std::decay_t<decltype(val)>>::value) {
+                        vstore(dst, val.hi);
+                        vstore(dst + ring_lo, val.lo);
+                    } else if constexpr (is_ophilo<std::decay_t<decltype(val)>>::value) {
+                        vstore(dst, val.op);
+                        vstore(dst + ring_lo, val.hi);
+                        vstore(dst + 2 * ring_lo, val.lo);
+                    } else {
+                        vstore(dst, val);
+                    }
+                }
+            };
+            prefetch(zlo - 1);
+            commit(0);
+            prefetch(zlo);
+            commit(1);
+            if (pipe) {
+                prefetch(zlo + 1);
+                own_of(zlo, opre);
+            }
+            for (int z = zlo; z < zhi; z += PL) {
+                const int np = min(PL, zhi - z);
+#pragma unroll
+                for (int q = 1; q <= PL; ++q) {
+                    if (q > np) break;
+                    if (!pipe || q > 1) prefetch(z + q);
+                    commit(slot(z + q));
+                }
+                plane_weights(z);   // (FINE_PLANES is 1)
+                __syncthreads();
+                Own cur[PL][KS];
+                if (pipe) {
+#pragma unroll
+                    for (int k = 0; k < KS; ++k) cur[0][k] = opre[k];
+#pragma unroll
+                    for (int q = 1; q < PL; ++q)
+                        if (q < np) own_of(z + q, cur[q]);
+                    if (z + np < zhi) {
+                        prefetch(z + np + 1);
+                        own_of(z + np, opre);
+                    }
+                } else {
+#pragma unroll
+                    for (int q = 0; q < PL; ++q)
+                        if (q < np) own_of(z + q, cur[q]);
+                }
+#pragma unroll
+                for (int q = 0; q < PL; ++q) {
+                    if (q >= np) break;
+                    const int zq = z + q;
+                    const int sc = slot(zq), sp = slot(zq + 1), sm = slot(zq - 1);
+                    plane_terms(zq);
+#pragma unroll
+                    for (int k = 0; k < KS; ++k) {
+                        const int rr = ty + k * RP;
+                        if (rr >= TY) continue;
+                        out(zq * n2 + (y0 + rr) * n + x0, k, y0 + rr, cur[q][k], ring + (sc * RW + rr + 1) * n,
+                            ring + (sp * RW + rr + 1) * n, ring + (sm * RW + rr + 1) * n);
+                    }
+                }
+            }
+            __syncthreads();   // the next tile's prologue rewrites slots 0 and 1
+        }
+    };
+    // ---- pointwise loop over owned points, one plane of KS rows at a time
+    auto owned = [&](auto&& load, auto&& fn) {
+        using Raw = decltype(load(0));
+        for (int tt = t_lo; tt < t_hi; ++tt) {
+            int y0, zlo, zhi;
+            geo.tile(tt, y0, zlo, zhi);
+            for (int z = zlo; z < zhi; ++z) {
+                Raw v[KS];
+#pragma unroll
+                for (int k = 0; k < KS; ++k)
+                    if (ty + k * RP < TY) v[k] = load(z * n2 + (y0 + ty + k * RP) * n + x0);
+#pragma unroll
+                for (int k = 0; k < KS; ++k)
+                    if (ty + k * RP < TY) fn(z * n2 + (y0 + ty + k * RP) * n + x0, v[k]);
+            }
+        }
+    };
+    // The 7-point operand values of the W points from ring rows (vector loads).
+    auto nb7 = [&](const auto* rowc, const auto* rowzp, const auto* rowzm) {
+        using T = std::remove_const_t<std::remove_pointer_t<decltype(rowc)>>;
+        Nb7<T, W> o;
+        o.c = vload<T, W>(rowc + x0);
+        shift(rowc, o.c, o.xp, o.xm);
+        o.yp = vload<T, W>(rowc + n + x0);
+        o.ym = vload<T, W>(rowc - n + x0);
+        o.zp = vload<T, W>(rowzp + x0);
+        o.zm = vload<T, W>(rowzm + x0);
+        return o;
+    };
+    // The stored perturbation at the W points from index i (FINE_MODE_IMPLICIT_PERT).  It is
+    // loaded where the stencil uses it, not one plane ahead with the other owned-point
+    // inputs: its 3 W registers held across the march made the instantiation spill.
+    auto load_pert = [&](int i) -> PertV<KT, W, PT> {
+        PertV<KT, W, PT> o;
+        if constexpr (PT) {
+            o.x = vload<KT, W>(bpk + i);
+            o.y = vload<KT, W>(bpk + Ng + i);
+            o.z = vload<KT, W>(bpk + 2 * Ng + i);
+        }
+        return o;
+    };
+    // FP64: the six neighbours' weights at the W points of row slot k in plane z
+    struct W6 { Vec<KT, W> xp, xm, yp, ym, zp, zm; };
+    auto weights = [&](int k, int z, const PertV<KT, W, PT>& pb) -> W6 {
+        W6 o;
+        const double* wr = reinterpret_cast<const double*>(wz) + (ty + k * RP) * n + x0;
+        const double* yr = reinterpret_cast<const double*>(wy) + (z & 1) * 2 * n + x0;
+        const KT ax = kx_y[k] + kx_z, axp = ax - c1, axm = -(ax + c1);
+#pragma unroll
+        for (int e = 0; e < W; ++e) {
+            o.xp.v[e] = axp;
+            o.xm.v[e] = axm;
+            o.yp.v[e] = (KT)yr[e];
+            o.ym.v[e] = (KT)yr[n + e];
+            o.zp.v[e] = (KT)wr[e];
+            o.zm.v[e] = (KT)wr[TY * n + e];
+            if constexpr (PT) {
+                const KT sx = kp * pb.x.v[e], sy = kp * pb.y.v[e], sz = kp * pb.z.v[e];
+                o.xp.v[e] += sx, o.xm.v[e] -= sx;
+                o.yp.v[e] += sy, o.ym.v[e] -= sy;
+                o.zp.v[e] += sz, o.zm.v[e] -= sz;
+            }
+        }
+        return o;
+    };
+    // A = I + dt L at the W points of row slot k (pb: the perturbation there)
+    auto applyA = [&](int k, const Vec<KT, W>& c, const Vec<KT, W>& xp, const Vec<KT, W>& xm,
+                      const Vec<KT, W>& yp, const Vec<KT, W>& ym, const Vec<KT, W>& zp,
+                      const Vec<KT, W>& zm, const PertV<KT, W, PT>& pb) -> Vec<KT, W> {
+        if constexpr (WT) {
+            const W6 w = weights(k, zcur, pb);
+            Vec<KT, W> v;
+#pragma unroll
+            for (int e = 0; e < W; ++e)
+                v.v[e] = c0 * c.v[e] + w.xp.v[e] * xp.v[e] + w.xm.v[e] * xm.v[e] + w.yp.v[e] * yp.v[e] +
+                         w.ym.v[e] * ym.v[e] + w.zp.v[e] * zp.v[e] + w.zm.v[e] * zm.v[e];
+            return v;
+        }
+        Vec<KT, W> o;
+#pragma unroll
+        for (int e = 0; e < W; ++e) {
+            KT ax = kx_y[k] + kx_z;
+            KT ay = ky_x[e] + ky_z;
+            KT az = kz_x[e] + kz_y[k];
+            if constexpr (PT) {
+                ax += kp * pb.x.v[e];
+                ay += kp * pb.y.v[e];
+                az += kp * pb.z.v[e];
+            }
+            o.v[e] = c0 * c.v[e] + (ax - c1) * xp.v[e] - (ax + c1) * xm.v[e] + (ay - c1) * yp.v[e] -
+                     (ay + c1) * ym.v[e] + (az - c1) * zp.v[e] - (az + c1) * zm.v[e];
+        }
+        return o;
+    };
+    using VK = Vec<KT, W>;
+    using VD = Vec<double, W>;
     // Sums of a phase's dot products over the group, then post(sums) in thread 0, and the
     // barrier between phases; false: the barrier gave up.
     auto finish = [&](auto& acc, auto&& post) -> bool {
@@ -722,42 +997,46 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
                           return o;
                       },
                       [&](int) -> NoOwn { return NoOwn{}; },
-                      [&](int i, int, int y, const NoOwn&, const double* rowc, const double* rowzp,
+                      [&](int i, int k, int y, const NoOwn&, const double* rowc, const double* rowzp,
                           const double* rowzm) {
-                          const int z = i / n2;
-                          const double bx = tabd[TXY * n + y] + tabd[TXZ * n + z];
-                          const double byz = tabd[TYZ * n + z], bzy = tabd[TZY * n + y];
                           // one point at a time: the FP64 stencil of all W points at once
-                          // would raise the register count of the whole kernel
+                          // would raise the register count of the whole kernel.  dt L u from
+                          // differences to the centre (the weights of L add up to zero), so
+                          // its rounding scales with the differences.
+                          const double ax = kx_y[k] + kx_z, axp = ax - c1, axm = -(ax + c1);
+                          const double* wr = wz + (ty + k * RP) * n;
+                          const double* yr = wy + (zcur & 1) * 2 * n;
+                          const double dtd = dt;
 #pragma unroll 1
                           for (int e = 0; e < W; ++e) {
                               const int x = x0 + e;
                               const int xp = (e == W - 1) ? xr : x + 1;
                               const int xm = (e == 0) ? xl : x - 1;
                               const double c = rowc[x];
-                              const double uxp = rowc[xp], uxm = rowc[xm];
-                              const double uyp = rowc[n + x], uym = rowc[x - n];
-                              const double uzp = rowzp[x], uzm = rowzm[x];
-                              double bxe = bx;
-                              double by = tabd[TYX * n + x] + byz;
-                              double bz = tabd[TZX * n + x] + bzy;
+                              double wxp = axp, wxm = axm, wyp = yr[x], wym = yr[n + x], wzp = wr[x], wzm = wr[TY * n + x];
                               if constexpr (PT) {
                                   const double* bpd = reinterpret_cast<const double*>(bpk);
-                                  bxe += bpd[i + e];
-                                  by += bpd[Ng + i + e];
-                                  bz += bpd[2 * Ng + i + e];
+                                  const double sx = kp * bpd[i + e], sy = kp * bpd[Ng + i + e], sz = kp * bpd[2 * Ng + i + e];
+                                  wxp += sx, wxm -= sx;
+                                  wyp += sy, wym -= sy;
+                                  wzp += sz, wzm -= sz;
                               }
-                              const double adv = bxe * (uxp - uxm) + by * (uyp - uym) + bz * (uzp - uzm);
-                              const double lap = (uxp + uxm) + (uyp + uym) + (uzp + uzm) - 6.0 * c;
-                              const double Lu = adv * inv2h - epsh2 * lap;
-                              double fi = fp ? fp[i + e] : 0.0;
-                              if (tdep) fi += ftd[x] + ftd[n + y] + ftd[2 * n + z];
-                              const KT rk = (KT)(dt * (fi - Lu));
+                              const double dLu = wxp * (rowc[xp] - c) + wxm * (rowc[xm] - c) + wyp * (rowc[n + x] - c) +
+                                                 wym * (rowc[x - n] - c) + wzp * (rowzp[x] - c) + wzm * (rowzm[x] - c);
+                              KT rk;
+                              double bi = c;
+                              if (fp || tdep) {
+                                  double fi = fp ? fp[i + e] : 0.0;
+                                  if (tdep) fi += ftd[x] + ftd[n + y] + ftd[2 * n + zcur];
+                                  rk = (KT)(dtd * fi - dLu);
+                                  bi += dtd * fi;
+                              } else {
+                                  rk = (KT)(-dLu);
+                              }
                               if (Wt) Wt[i + e] = c;
                               if (snap_j) snap_j[i + e] = c;
                               r[i + e] = rk;
                               rh[i + e] = rk;
-                              const double bi = c + dt * fi;
                               acc.f[0] += rk * rk;
                               acc.f[1] += (KT)(bi * bi);
                           }
@@ -887,11 +1166,297 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
             })) return;
             const bool conv = sh.flag != 0;
             int it = 0;
-#define FINE_GIVE_UP
-#define FINE_PIPE true
-#include "fine_bicgstab.inl"
-#undef FINE_PIPE
-#undef FINE_GIVE_UP
+            while (!conv) {
+                ++it;
+                const bool first = it == 1;
+                // ---------------- ph1: p = r + beta (p' - omega v'), v = A p
+                KT* pn = (it & 1) ? p1 : p0;
+                KT* po = (it & 1) ? p0 : p1;
+                KT* vn = (it & 1) ? v1 : v0;
+                KT* vo = (it & 1) ? v0 : v1;
+                {
+                    const KT bk = (KT)sh.beta, ok = (KT)sh.omega;
+                    Acc<KT, 1> acc;
+                    acc.init();
+                    march(true, ringk,
+                          [&](int i) -> RawP<KT, W> {
+                              RawP<KT, W> o;
+                              o.r = vload<KT, W>(r + i);
+                              if (!first) {
+                                  o.p = vload<KT, W>(po + i);
+                                  o.v = vload<KT, W>(vo + i);
+                              } else {
+#pragma unroll
+                                  for (int e = 0; e < W; ++e) { o.p.v[e] = (KT)0; o.v.v[e] = (KT)0; }
+                              }
+                              return o;
+                          },
+                          [&](const RawP<KT, W>& v) -> VK {
+                              VK o;
+#pragma unroll
+                              for (int e = 0; e < W; ++e)
+                                  o.v[e] = !DF && first ? v.r.v[e] : v.r.v[e] + bk * (v.p.v[e] - ok * v.v.v[e]);
+                              return o;
+                          },
+                          [&](int i) -> OwnH<KT, W, PT> { return {vload<KT, W>(rh + i), {}}; },
+                          [&](int i, int k, int, const OwnH<KT, W, PT>& ow, const KT* rowc, const KT* rowzp,
+                              const KT* rowzm) {
+                              const VK& rhv = ow.h;
+                              const auto q7 = nb7(rowc, rowzp, rowzm);
+                              const VK av = applyA(k, q7.c, q7.xp, q7.xm, q7.yp, q7.ym, q7.zp, q7.zm, load_pert(i));
+                              vstore(pn + i, q7.c);
+                              vstore(vn + i, av);
+#pragma unroll
+                              for (int e = 0; e < W; ++e) acc.f[0] += rhv.v[e] * av.v[e];
+                              acc.tick();
+                          });
+                    if (!finish(acc, [&](const double* s) {
+                    const double rv = s[0];
+                    if (rv == 0.0 || !isfinite(rv)) {
+                        sh.status = isfinite(rv) ? DERR_BREAKDOWN : DERR_NONFINITE;
+                        sh.flag = 1;
+                    } else {
+                        sh.alpha = sh.rho / rv;
+                        sh.flag = 0;
+                    }
+                    })) return;
+                }
+                if (sh.flag) {
+                    --it;
+                    break;
+                }
+                // ---------------- ph2: s = r - alpha v, t = A s
+                {
+                    const KT al = (KT)sh.alpha;
+                    // FP64: <rhat, t> too, from which beta and the stopping test follow without
+                    // the products of the update pass: <rhat, s> = rho - alpha <rhat, v> is zero
+                    // up to rounding, so <rhat, r> = -omega <rhat, t>, and ||r||^2 = <s,s> - omega <t,s>
+                    constexpr int NQ2 = DF ? 3 : 4;
+                    Acc<KT, NQ2> acc;
+                    acc.init();
+                    march(true, ringk,
+                          [&](int i) -> RawS<KT, W> { return {vload<KT, W>(r + i), vload<KT, W>(vn + i)}; },
+                          [&](const RawS<KT, W>& v) -> VK {
+                              VK o;
+#pragma unroll
+                              for (int e = 0; e < W; ++e) o.v[e] = v.r.v[e] - al * v.v.v[e];
+                              return o;
+                          },
+                          [&](int i) -> std::conditional_t<DF, NoOwn, VK> {
+                              if constexpr (DF) return NoOwn{};
+                              else return vload<KT, W>((first ? pn : rh) + i);   // rhat is the first p
+                          },
+                          [&](int i, int k, int, const auto& hv, const KT* rowc, const KT* rowzp,
+                              const KT* rowzm) {
+                              const auto q7 = nb7(rowc, rowzp, rowzm);
+                              const VK tv = applyA(k, q7.c, q7.xp, q7.xm, q7.yp, q7.ym, q7.zp, q7.zm, load_pert(i));
+                              vstore(t + i, tv);
+#pragma unroll
+                              for (int e = 0; e < W; ++e) {
+                                  acc.f[0] += tv.v[e] * q7.c.v[e];
+                                  acc.f[1] += tv.v[e] * tv.v[e];
+                                  acc.f[2] += q7.c.v[e] * q7.c.v[e];
+                                  if constexpr (!DF) acc.f[3] += hv.v[e] * tv.v[e];
+                              }
+                              acc.tick();
+                          });
+                    if (!finish(acc, [&](const double* s) {
+                    const double ts = s[0], tt2 = s[1], ss = s[2];
+                    const int half = sqrt(ss) <= sh.thr;
+                    if (!half) {
+                        if (tt2 == 0.0 || !isfinite(tt2)) {
+                            sh.status = isfinite(tt2) ? DERR_BREAKDOWN : DERR_NONFINITE;
+                            sh.omega = 0.0;
+                        } else {
+                            sh.omega = ts / tt2;
+                            if (sh.omega == 0.0) sh.status = DERR_BREAKDOWN;
+                        }
+                    }
+                    sh.flag = half;
+                    if constexpr (!DF) {   // 0: go on, 1: delta += alpha p only, 2: the step is done
+                        if (!half && sh.status == 0) {
+                            const double rr1 = fma(-sh.omega, ts, ss), rho_new = -sh.omega * s[3];
+                            sh.flag = 2;
+                            if (!isfinite(rr1)) sh.status = DERR_NONFINITE;
+                            else if (sqrt(fmax(rr1, 0.0)) <= sh.thr) {}
+                            else if (rho_new == 0.0) sh.status = DERR_BREAKDOWN;
+                            else if (it >= J.maxit) sh.status = DERR_NOT_CONVERGED;
+                            else {
+                                sh.beta = (rho_new / sh.rho) * (sh.alpha / sh.omega);
+                                sh.rho = rho_new;
+                                sh.flag = 0;
+                            }
+                        } else {
+                            sh.flag = 1;
+                        }
+                    }
+                    })) return;
+                }
+                if constexpr (!DF) {
+                    // ---------------- ph3: delta += alpha p + omega s ; r = s - omega t if it goes on
+                    const int act = sh.flag;
+                    const KT al = (KT)sh.alpha, om = (KT)sh.omega;
+                    owned([&](int i) -> Raw6<KT, W> {
+                              Raw6<KT, W> o;
+                              if (!first) o.d = vload<KT, W>(delta + i);
+                              o.p = vload<KT, W>(pn + i);
+                              if (act != 1) {
+                                  o.r = vload<KT, W>(r + i);
+                                  o.v = vload<KT, W>(vn + i);
+                              }
+                              if (act == 0) o.t = vload<KT, W>(t + i);
+                              return o;
+                          },
+                          [&](int i, const Raw6<KT, W>& v) {
+                              VK dn, rn;
+#pragma unroll
+                              for (int e = 0; e < W; ++e) {
+                                  dn.v[e] = first ? al * v.p.v[e] : v.d.v[e] + al * v.p.v[e];
+                                  if (act != 1) {
+                                      const KT sc_ = v.r.v[e] - al * v.v.v[e];
+                                      dn.v[e] += om * sc_;
+                                      if (act == 0) rn.v[e] = sc_ - om * v.t.v[e];
+                                  }
+                              }
+                              vstore(delta + i, dn);
+                              if (act == 0) vstore(r + i, rn);
+                          });
+                    if (!group_barrier(bar, G, a.spin_limit, a.err)) return;
+                    if (act != 0) break;
+                    continue;
+                }
+                const bool half = sh.flag != 0;
+                // ---------------- ph3: delta += alpha p + omega s ; r = s - omega t
+                {
+                    const KT al = (KT)sh.alpha, om = (KT)sh.omega;
+                    const bool first = (it == 1) && !xg;   // delta holds the initial guess
+                    const bool upd_r = !half && sh.status == 0;
+                    Acc<KT, 2> acc;
+                    acc.init();
+                    // the update of the owned points from their six inputs
+                    auto p3_fn = [&](int i, const Raw6<KT, W>& v) {
+                        VK dn, rn;
+#pragma unroll
+                        for (int e = 0; e < W; ++e) {
+                            const KT sc_ = v.r.v[e] - al * v.v.v[e];
+                            dn.v[e] = v.d.v[e] + al * v.p.v[e] + om * sc_;
+                            rn.v[e] = sc_ - om * v.t.v[e];
+                            acc.f[0] += v.h.v[e] * rn.v[e];
+                            acc.f[1] += rn.v[e] * rn.v[e];
+                        }
+                        vstore(delta + i, dn);
+                        vstore(r + i, rn);
+                        acc.tick();
+                    };
+                    bool staged3 = false;
+                    if constexpr (DF && KS == 1) {
+                        if (upd_r) {
+                            // inputs of plane z staged by cp.async while planes z-2, z-1 are
+                            // updated; each thread reads back only what it copied, so no
+                            // barrier is needed; layout [slot][input][thread][W] (no bank
+                            // conflicts).  The ring is idle in this phase.
+                            staged3 = true;
+                            constexpr int NS = FINE_PH3_SLOTS;
+                            float* stg = reinterpret_cast<float*>(ring_raw);
+                            const int nthr = blockDim.x;
+                            const bool act = ty < TY;
+                            auto sad = [&](int sl, int q) { return stg + ((size_t)(sl * 6 + q) * nthr + threadIdx.x) * W; };
+                            for (int tt = t_lo; tt < t_hi; ++tt) {
+                                int y0, zlo, zhi;
+                                geo.tile(tt, y0, zlo, zhi);
+                                const int rowoff = (y0 + ty) * n + x0;
+                                auto issue = [&](int z, int sl) {
+                                    if (act && z < zhi) {
+                                        const long long i = (long long)z * n2 + rowoff;
+                                        if (!first) cp_async_b<4 * W>(sad(sl, 0), delta + i);
+                                        cp_async_b<4 * W>(sad(sl, 1), pn + i);
+                                        cp_async_b<4 * W>(sad(sl, 2), r + i);
+                                        cp_async_b<4 * W>(sad(sl, 3), vn + i);
+                                        cp_async_b<4 * W>(sad(sl, 4), t + i);
+                                        cp_async_b<4 * W>(sad(sl, 5), rh + i);
+                                    }
+                                    cp_async_commit_group();
+                                };
+#pragma unroll
+                                for (int d = 0; d < NS - 1; ++d) issue(zlo + d, d);
+                                int sl = 0;
+                                for (int z = zlo; z < zhi; ++z) {
+                                    // refill the slot of plane z - 1 (read last iteration)
+                                    issue(z + NS - 1, sl == 0 ? NS - 1 : sl - 1);
+                                    cp_async_wait_newest<NS - 1>();
+                                    if (act) {
+                                        Raw6<KT, W> v;
+                                        if (!first) v.d = vload<float, W>(sad(sl, 0));
+                                        else {
+#pragma unroll
+                                            for (int e = 0; e < W; ++e) v.d.v[e] = 0.0f;
+                                        }
+                                        v.p = vload<float, W>(sad(sl, 1));
+                                        v.r = vload<float, W>(sad(sl, 2));
+                                        v.v = vload<float, W>(sad(sl, 3));
+                                        v.t = vload<float, W>(sad(sl, 4));
+                                        v.h = vload<float, W>(sad(sl, 5));
+                                        p3_fn(z * n2 + rowoff, v);
+                                    }
+                                    sl = (sl + 1 == NS) ? 0 : sl + 1;
+                                }
+                                cp_async_wait_newest<0>();
+                            }
+                        }
+                    }
+                    if (upd_r && !staged3) {
+                        owned([&](int i) -> Raw6<KT, W> {
+                                  Raw6<KT, W> o;
+                                  if (!first) o.d = vload<KT, W>(delta + i);
+                                  else {
+#pragma unroll
+                                      for (int e = 0; e < W; ++e) o.d.v[e] = (KT)0;
+                                  }
+                                  o.p = vload<KT, W>(pn + i);
+                                  o.r = vload<KT, W>(r + i);
+                                  o.v = vload<KT, W>(vn + i);
+                                  o.t = vload<KT, W>(t + i);
+                                  o.h = vload<KT, W>(rh + i);
+                                  return o;
+                              },
+                              p3_fn);
+                    } else if (!upd_r) {
+                        owned([&](int i) -> RawP2<KT, W> {
+                                  RawP2<KT, W> o;
+                                  if (!first) o.d = vload<KT, W>(delta + i);
+                                  else {
+#pragma unroll
+                                      for (int e = 0; e < W; ++e) o.d.v[e] = (KT)0;
+                                  }
+                                  o.p = vload<KT, W>(pn + i);
+                                  return o;
+                              },
+                              [&](int i, const RawP2<KT, W>& v) {
+                                  VK dn;
+#pragma unroll
+                                  for (int e = 0; e < W; ++e) dn.v[e] = v.d.v[e] + al * v.p.v[e];
+                                  vstore(delta + i, dn);
+                              });
+                    }
+                    if (!finish(acc, [&](const double* s) {
+                        if (!upd_r) return;   // delta is final
+                        const double rho_new = s[0], rr1 = s[1];
+                        int stop = 1;
+                        if (!isfinite(rr1)) sh.status = DERR_NONFINITE;
+                        else if (sqrt(rr1) <= sh.thr) {}
+                        else if (rho_new == 0.0) sh.status = DERR_BREAKDOWN;
+                        else if (it >= J.maxit) sh.status = DERR_NOT_CONVERGED;
+                        else {
+                            sh.beta = (rho_new / sh.rho) * (sh.alpha / sh.omega);
+                            sh.rho = rho_new;
+                            stop = 0;
+                        }
+                        sh.flag = stop;
+                    })) return;
+                    if (!upd_r) break;
+                        }
+                if (sh.flag) break;
+            }
             dvalid = it > 0 || xg;
             its_total += it;
             its_max = max(its_max, it);
@@ -962,7 +1527,8 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
 }
 
 // ------------------------------------------------------------------------------------
-// Launch geometry.  W = 4 points per thread when n % 4 == 0, else 1.  A row has n/W
+// Launch geometry.  W = 4 points per thread (2 in FP64, where four points' operands spill at
+// the 128 registers of two 256-thread CTAs an SM) when n % 4 == 0, else 1.  A row has n/W
 // lanes.  CTAs of at most 128 threads (RP rows a pass, one owned row a thread) when the
 // tile keeps at least 8 rows: the kernel is latency-bound at 128 registers a thread, and
 // small CTAs (4 an SM) let the groups of a launch fill nearly every CTA slot (64^3, 64
@@ -977,7 +1543,7 @@ struct FineGeom {
 
 inline FineGeom fine_geom(int n, bool fp32) {
     FineGeom g{};
-    g.W = (n % 4 == 0) ? 4 : 1;
+    g.W = (n % 4 == 0) ? (fp32 ? 4 : 2) : 1;
     g.lanes = n / g.W;
     int rp128 = 1;
     for (int rp = 1; rp <= n; ++rp)
@@ -986,9 +1552,9 @@ inline FineGeom fine_geom(int n, bool fp32) {
     for (int rp = 1; rp <= n; ++rp)
         if (n % rp == 0 && rp * g.lanes <= 256) g.RP = rp;
     g.KS = 1;
-    if (rp128 >= 8) {
+    if (rp128 >= (g.W == 2 ? 4 : 8)) {
         g.RP = rp128;
-    } else if (n % (2 * g.RP) == 0 && 2 * g.RP <= 16 &&
+    } else if (!(g.W == 2 && g.RP >= 4) && n % (2 * g.RP) == 0 && 2 * g.RP <= 16 &&
                (size_t)FINE_SLOTS * (2 * g.RP + 2) * n * 8 <= 64 * 1024) {
         g.KS = 2;
     }
@@ -1001,8 +1567,10 @@ inline FineGeom fine_geom(int n, bool fp32) {
     const size_t ring = (size_t)FINE_SLOTS * (g.TY + 2) * n * (fp32 ? 12 : 8);
     // FP32 mode, one owned row a thread: the pointwise phase stages FINE_PH3_SLOTS planes of
     // six float inputs per thread over the ring
+    // FP64: the weights of the z neighbours of a tile plane and of the y neighbours of two planes
+    const size_t wts = fp32 ? 0 : (size_t)(2 * g.TY * n + 4 * n) * sizeof(double);
     const size_t ph3 = (fp32 && g.KS == 1) ? (size_t)FINE_PH3_SLOTS * 6 * g.threads * g.W * sizeof(float) : 0;
-    g.smem = tabs + std::max(ring, ph3);
+    g.smem = tabs + std::max(ring, ph3) + wts;
     return g;
 }
 

@@ -19,7 +19,7 @@ static FineFn pick_pert(int KF, int KS) {
 
 FineFn fine_fn_pert(bool fp32, int W, int KF, int KS) {
     if (fp32) return W == 4 ? pick_pert<float, 4>(KF, KS) : pick_pert<float, 1>(KF, KS);
-    return W == 4 ? pick_pert<double, 4>(KF, KS) : pick_pert<double, 1>(KF, KS);
+    return W == 2 ? pick_pert<double, 2>(KF, KS) : pick_pert<double, 1>(KF, KS);
 }
 
 }  // namespace pr
