@@ -192,14 +192,15 @@ cudaError_t launch_to_float(const double* in, float* out, long long n, cudaStrea
 // ------------------------------------------------------------------------------------
 // out = L u or L^T u on whole grid functions.  Every supported velocity has b_d
 // independent of x_d, so b_d(x +- e_d) = b_d(x) and L^T only flips the advection sign.
-// One thread per point runs over all columns of its batch item: the neighbour offsets and
+// One thread per point runs over all columns of `per` batch items: the neighbour offsets and
 // the velocity terms are formed once (32-bit index arithmetic, no FP64 division), each
-// column costs its seven loads and a dozen FP64 operations.
+// column costs its seven loads and 13 FP64 operations.  The FP64 pipe (2 operations a cycle
+// and SM) bounds it: with one item a thread, forming the terms for each of 32 single-column
+// items at 128^3 took as many operations again, 2.93 -> 1.69 ms (13 operations a point alone take 1.43 ms).
 template <typename TI, typename TO>
 __global__ void __launch_bounds__(256) apply_L_kernel(Grid g, const void* const* in_cols, void* const* out_cols,
                                                       const int* count, int ldcols, bool transpose,
-                                                      double inv2h, double epsh2) {
-    const int b = blockIdx.y;
+                                                      double inv2h, double epsh2, int per, int B) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int)g.Ng) return;
     const int n = g.n, n2 = n * n;
@@ -234,21 +235,24 @@ __global__ void __launch_bounds__(256) apply_L_kernel(Grid g, const void* const*
         cyp = -inv2h * (by + g.pert[N + iyp]), cym = inv2h * (by + g.pert[N + iym]);
         czp = -inv2h * (bz + g.pert[2 * N + izp]), czm = inv2h * (bz + g.pert[2 * N + izm]);
     }
-    const int cnt = count[b];
-    for (int c = 0; c < cnt; ++c) {
-        const TI* in = (const TI*)in_cols[(size_t)b * ldcols + c];
-        TO* out = (TO*)out_cols[(size_t)b * ldcols + c];
-        const double u0 = (double)in[i];
-        const double uxp = (double)in[ixp], uxm = (double)in[ixm];
-        const double uyp = (double)in[iyp], uym = (double)in[iym];
-        const double uzp = (double)in[izp], uzm = (double)in[izm];
-        double adv;
-        if (!(transpose && g.pert))   // cd_m = -cd_p: differences first, exact for close values
-            adv = cxp * (uxp - uxm) + cyp * (uyp - uym) + czp * (uzp - uzm);
-        else
-            adv = (cxp * uxp + cxm * uxm) + (cyp * uyp + cym * uym) + (czp * uzp + czm * uzm);
-        const double lap = (uxp + uxm) + (uyp + uym) + (uzp + uzm) - 6.0 * u0;
-        out[i] = (TO)(adv - epsh2 * lap);
+    const int b1 = min(B, ((int)blockIdx.y + 1) * per);
+    for (int b = blockIdx.y * per; b < b1; ++b) {
+        const int cnt = count[b];
+        for (int c = 0; c < cnt; ++c) {
+            const TI* in = (const TI*)in_cols[(size_t)b * ldcols + c];
+            TO* out = (TO*)out_cols[(size_t)b * ldcols + c];
+            const double u0 = (double)in[i];
+            const double uxp = (double)in[ixp], uxm = (double)in[ixm];
+            const double uyp = (double)in[iyp], uym = (double)in[iym];
+            const double uzp = (double)in[izp], uzm = (double)in[izm];
+            double adv;
+            if (!(transpose && g.pert))   // cd_m = -cd_p: differences first, exact for close values
+                adv = cxp * (uxp - uxm) + cyp * (uyp - uym) + czp * (uzp - uzm);
+            else
+                adv = (cxp * uxp + cxm * uxm) + (cyp * uyp + cym * uym) + (czp * uzp + czm * uzm);
+            const double lap = (uxp + uxm) + (uyp + uym) + (uzp + uzm) - 6.0 * u0;
+            out[i] = (TO)(adv - epsh2 * lap);
+        }
     }
 }
 
@@ -321,17 +325,24 @@ cudaError_t launch_apply_L(const Grid& g, const void* const* in_cols, void* cons
                            bool out_f32, bool transpose, cudaStream_t st) {
     if (max_count <= 0 || B <= 0) return cudaSuccess;
     if (g.Ng > (1LL << 30)) return cudaErrorInvalidValue;   // 32-bit point indices
-    dim3 grid((unsigned)((g.Ng + 255) / 256), (unsigned)B);
+    // items a thread: as many as leave every SM 16 blocks (two rounds of 8)
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const long long bx = (g.Ng + 255) / 256;
+    const int per = (int)std::max<long long>(1, std::min<long long>(B, bx * B / (16LL * std::max(1, sms))));
+    dim3 grid((unsigned)bx, (unsigned)((B + per - 1) / per));
     const double inv2h = 0.5 / g.h, epsh2 = g.eps / (g.h * g.h);
     if (in_f32 && out_f32)
-        apply_L_kernel<float, float><<<grid, 256, 0, st>>>(g, in_cols, out_cols, count, ldcols, transpose, inv2h, epsh2);
+        apply_L_kernel<float, float><<<grid, 256, 0, st>>>(g, in_cols, out_cols, count, ldcols, transpose, inv2h, epsh2, per, B);
     else if (in_f32)
-        apply_L_kernel<float, double><<<grid, 256, 0, st>>>(g, in_cols, out_cols, count, ldcols, transpose, inv2h, epsh2);
+        apply_L_kernel<float, double><<<grid, 256, 0, st>>>(g, in_cols, out_cols, count, ldcols, transpose, inv2h, epsh2, per, B);
     else if (out_f32)
-        apply_L_kernel<double, float><<<grid, 256, 0, st>>>(g, in_cols, out_cols, count, ldcols, transpose, inv2h, epsh2);
+        apply_L_kernel<double, float><<<grid, 256, 0, st>>>(g, in_cols, out_cols, count, ldcols, transpose, inv2h, epsh2, per, B);
     else
         apply_L_kernel<double, double><<<grid, 256, 0, st>>>(g, in_cols, out_cols, count, ldcols, transpose, inv2h,
-                                                             epsh2);
+                                                             epsh2, per, B);
     ++g_launch_count;
     return cudaGetLastError();
 }
