@@ -1,6 +1,6 @@
 // POD of snapshot matrices (Algorithm 1, POD_Mode, and the two-level POD of Case II):
 //   Gram W^T M W (M = I)           -> gram_kernel     (batched, split over points)
-//   eigenpairs, rank r, dimension m -> eig_pod_kernel  (cyclic Jacobi, FP64, one CTA/matrix)
+//   eigenpairs, rank r, dimension m -> eig_pod_kernel  (eig.cu: cyclic Jacobi, FP64)
 //   R = W Y_m Lambda_m^{-1/2}       -> tsmm_kernel     (tall-skinny multiply)
 //   Cholesky-QR re-orthonormalisation -> gram + chol_inv_kernel + tsmm, one pass
 // The Gram and projection stream every snapshot once per use; the small dense steps stay
@@ -639,202 +639,6 @@ cudaError_t launch_tsmm(const TsmmArgs& a, bool in_f32, bool out_f32, cudaStream
     } else {
         tsmm_kernel<double, double, double><<<grid, 256, cells * sizeof(double), st>>>(a);
     }
-    ++g_launch_count;
-    return cudaGetLastError();
-}
-
-// ------------------------------------------------------------------------------------
-// Batched symmetric eigensolver (parallel cyclic Jacobi, round-robin pairing) + POD
-// selection of Algorithm 1.
-constexpr int EIG_THREADS = 256;
-constexpr int EIG_MAX_SWEEPS = 40;
-
-__device__ __forceinline__ void rr_pair(int r, int i, int Kp, int& p, int& q) {
-    const int M = Kp - 1;
-    if (i == 0) {
-        p = M;
-        q = r;
-    } else {
-        p = (r + i) % M;
-        q = (r - i + M) % M;
-    }
-}
-
-__global__ void __launch_bounds__(EIG_THREADS) eig_pod_kernel(EigArgs a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int b = blockIdx.x;
-    const int K = a.K[b];
-    double* lam_out = a.lam + (size_t)b * a.maxK;
-    double* Cb = a.C + (size_t)b * a.ldC_b;
-    if (K <= 0) {
-        if (threadIdx.x == 0) a.m[b] = 0;
-        return;
-    }
-    const int Kp = K + (K & 1);
-    const int ld = Kp + 1;   // odd stride in doubles: row and column sweeps hit distinct banks
-    double* A = reinterpret_cast<double*>(smem_raw);
-    double* V = A + (size_t)Kp * ld;
-    double* cs = V + (size_t)Kp * ld;           // [Kp/2][2]
-    double* lam = cs + Kp;                       // [Kp]
-    int* perm = reinterpret_cast<int*>(lam + Kp);  // [Kp]
-    int* pq = perm + Kp;                         // [Kp/2][2]: the round's pairs
-    __shared__ double red[32];
-    __shared__ int s_stop;
-    __shared__ double s_prev;   // ||off||_F^2 before the previous sweep
-    const double* Gb = a.G + (size_t)b * a.ldG_b;
-    for (int e = threadIdx.x; e < Kp * Kp; e += blockDim.x) {
-        const int i = e / Kp, j = e - i * Kp;
-        A[i * ld + j] = (i < K && j < K) ? Gb[(size_t)i * a.ldG + j] : 0.0;
-        V[i * ld + j] = (i == j) ? 1.0 : 0.0;
-    }
-    __syncthreads();
-    const int npair = Kp / 2;
-    // fixed thread -> (pair, first row) map of the rotation updates: no divisions per element
-    const int ti = threadIdx.x % npair, kst = blockDim.x / npair;
-    const int tk0 = threadIdx.x / npair;
-    for (int sweep = 0; sweep < EIG_MAX_SWEEPS; ++sweep) {
-        // convergence: off-diagonal Frobenius norm against the whole matrix
-        double off = 0.0, tot = 0.0;
-        for (int e = threadIdx.x; e < K * K; e += blockDim.x) {
-            const int i = e / K, j = e - i * K;
-            const double v = A[i * ld + j];
-            tot += v * v;
-            if (i != j) off += v * v;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            off += __shfl_down_sync(0xffffffffu, off, o);
-            tot += __shfl_down_sync(0xffffffffu, tot, o);
-        }
-        if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5] = off; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double so = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) so += red[w];
-            red[31] = so;
-        }
-        __syncthreads();
-        const double offsum = red[31];
-        __syncthreads();
-        if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5] = tot; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double st = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) st += red[w];
-            // converged when the off-diagonal part is at the rounding level of the Gram
-            // matrix itself, ||off||_F <= K eps ||A||_F: a tighter bound sits below the
-            // noise of the rotations (fused multiply-adds) and would never be met.  The
-            // rotations' own noise can also sit just above that bound, so a sweep that no
-            // longer cuts ||off|| four-fold within 16 times of it ends the iteration too
-            // (past the quadratic phase further sweeps only reshuffle rounding noise)
-            const double tolK = (double)K * 2.220446049250313e-16;
-            const bool stalled = sweep > 0 && offsum <= 256.0 * tolK * tolK * st && offsum * 16.0 >= s_prev;
-            s_stop = (offsum <= tolK * tolK * st) || st == 0.0 || stalled;
-            s_prev = offsum;
-        }
-        __syncthreads();
-        if (s_stop) break;
-        for (int r = 0; r < Kp - 1; ++r) {
-            for (int i = threadIdx.x; i < npair; i += blockDim.x) {
-                int p, q;
-                rr_pair(r, i, Kp, p, q);
-                double c = 1.0, s = 0.0;
-                if (p < K && q < K) {
-                    const double apq = A[p * ld + q];
-                    const double app = A[p * ld + p], aqq = A[q * ld + q];
-                    if (apq != 0.0 && fabs(apq) > 1e-300) {
-                        const double tau = (aqq - app) / (2.0 * apq);
-                        const double tt = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-                        c = 1.0 / sqrt(1.0 + tt * tt);
-                        s = tt * c;
-                    }
-                }
-                cs[2 * i] = c;
-                cs[2 * i + 1] = s;
-                pq[2 * i] = p;
-                pq[2 * i + 1] = q;
-            }
-            __syncthreads();
-            const bool upd = tk0 < kst && cs[2 * ti + 1] != 0.0;
-            const double c = cs[2 * ti], s = cs[2 * ti + 1];
-            const int p = pq[2 * ti], q = pq[2 * ti + 1];
-            if (upd) {
-                // A <- A J, V <- V J (columns p, q)
-                for (int k = tk0; k < Kp; k += kst) {
-                    const double akp = A[k * ld + p], akq = A[k * ld + q];
-                    A[k * ld + p] = c * akp - s * akq;
-                    A[k * ld + q] = s * akp + c * akq;
-                    const double vkp = V[k * ld + p], vkq = V[k * ld + q];
-                    V[k * ld + p] = c * vkp - s * vkq;
-                    V[k * ld + q] = s * vkp + c * vkq;
-                }
-            }
-            __syncthreads();
-            if (upd) {
-                // A <- J^T A (rows p, q)
-                for (int k = tk0; k < Kp; k += kst) {
-                    const double apk = A[p * ld + k], aqk = A[q * ld + k];
-                    A[p * ld + k] = c * apk - s * aqk;
-                    A[q * ld + k] = s * apk + c * aqk;
-                }
-            }
-            __syncthreads();
-        }
-    }
-    // eigenvalues, descending order (ties by index)
-    for (int i = threadIdx.x; i < K; i += blockDim.x) lam[i] = A[i * ld + i];
-    __syncthreads();
-    for (int i = threadIdx.x; i < K; i += blockDim.x) {
-        int rank = 0;
-        const double li = lam[i];
-        for (int j = 0; j < K; ++j) {
-            const double lj = lam[j];
-            rank += (lj > li) || (lj == li && j < i);
-        }
-        perm[rank] = i;
-    }
-    __syncthreads();
-    __shared__ int s_m;
-    if (threadIdx.x == 0) {
-        const double l1 = lam[perm[0]];
-        int m = 0;
-        if (l1 > 0.0) {
-            int r = 0;
-            for (int i = 0; i < K; ++i) r += lam[perm[i]] > a.tau * l1;
-            double total = 0.0;
-            for (int i = 0; i < r; ++i) total += sqrt(lam[perm[i]]);
-            double cum = 0.0;
-            m = r;
-            for (int i = 0; i < r; ++i) {
-                cum += sqrt(lam[perm[i]]);
-                if (cum >= a.gamma * total) { m = i + 1; break; }
-            }
-            if (a.cap > 0) m = min(m, a.cap);
-            m = min(m, r);
-        }
-        s_m = m;
-        a.m[b] = m;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < a.maxK; i += blockDim.x) lam_out[i] = (i < K) ? lam[perm[i]] : 0.0;
-    const int m = s_m;
-    for (int e = threadIdx.x; e < K * m; e += blockDim.x) {
-        const int i = e / m, j = e - i * m;
-        const int src = perm[j];
-        Cb[(size_t)i * a.ldC + j] = V[i * ld + src] / sqrt(lam[src]);
-    }
-}
-
-cudaError_t launch_eig_pod(const EigArgs& a, cudaStream_t st) {
-    if (a.B <= 0) return cudaSuccess;
-    const int Kp = a.maxK + (a.maxK & 1);
-    const size_t smem = (size_t)2 * Kp * (Kp + 1) * sizeof(double) + (size_t)2 * Kp * sizeof(double) +
-                        (size_t)2 * Kp * sizeof(int) + 16;
-    static size_t configured = 0;
-    if (smem > 48 * 1024 && smem > configured) {
-        cudaFuncSetAttribute(eig_pod_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        configured = smem;
-    }
-    eig_pod_kernel<<<a.B, EIG_THREADS, smem, st>>>(a);
     ++g_launch_count;
     return cudaGetLastError();
 }
