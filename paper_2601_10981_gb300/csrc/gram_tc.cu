@@ -21,22 +21,23 @@
 // those with s + t = c + 1, from at most four (s, t) pairs each.  Every 1024 points
 // (4 x 1024 x 2^12 = 2^24) the eight tiles (c = 2..9, all pairs with s + t <= 9; the
 // dropped ones weigh below 2^-58 of a leading product) are read back with tcgen05.ld and
-// added into FP64 accumulators with their weights, which are powers of two.  The only
-// roundings are those FP64 additions and the 56-bit truncation of each value, so the
-// result has the accuracy of an FP64 Gram.
+// added, with their weights, into exact 96-bit integers, which are rounded once a chunk.
+// The only other rounding is the 56-bit truncation of each value, so the result has the
+// accuracy of an FP64 Gram.
 //
 // Two forms share the digit scheme: the wide one described here (up to 64 columns,
 // gram_tc_kernel) and a narrow, warp-specialised one for up to 32 columns
 // (gram_tc32_kernel, described at its definition), which sums exactly and rounds once.
 //
-// Wide form.  Work split: a persistent grid, one CTA per SM (the eight tiles fill the SM's 512 TMEM
+// Wide form.  A persistent grid, one CTA per SM (the eight tiles fill the SM's 512 TMEM
 // columns); a CTA takes work units (batch item, chunk of points) in turn and, per stage
-// of 64 points, its 128 threads load the FP64 values, cut them into digits and store them
-// in shared memory in the canonical K-major layout of the MMA operands (8 x 16-byte core
-// matrices, no swizzle), then one thread issues the 80 MMAs of the stage and commits
-// them to an mbarrier.  Every wait on the mbarrier is bounded: on time-out the kernel
-// records PR_ERR_TIMEOUT, waits (bounded) for its MMAs in flight, frees its tensor memory
-// and returns.  Column maxima come from a pre-pass (colmax_kernel).
+// of 64 points, 512 threads cut eight values each (loaded a stage ahead) into digits and
+// store them into a ring of two stages in the MMA operands' layout; a seventeenth warp issues the MMAs.  Slices
+// follow one another in a stage, so one B operand spans four of them (N = 256) and a K-step
+// is six MMAs.  Every wait on an mbarrier is bounded: on time-out the kernel records
+// PR_ERR_TIMEOUT, waits (bounded) for its MMAs in flight, frees its tensor memory and
+// returns.  Column maxima come from a pre-pass (colmax_kernel).
+// TCFIG
 #include "pr_internal.cuh"
 
 #include <cuda_bf16.h>
@@ -48,44 +49,51 @@ namespace pr {
 
 namespace {
 
-constexpr int TC_THREADS = 256;   // 8 warps: two cover each tensor-memory lane quarter
+constexpr int TC_PROD = 512;          // producer threads: four warps for each tensor-memory lane quarter
+constexpr int TC_THREADS = TC_PROD + 32;   // + the MMA warp
 constexpr int TC_N = 64;             // columns handled (K <= 64)
 constexpr int TC_PTS = 64;           // points per shared-memory stage
 constexpr int TC_SLICES = 8;         // digits per value
 constexpr int TC_TILES = 8;          // accumulator tiles c = 2..9
-constexpr int TC_STAGES_PER_DRAIN = 16;   // 16 x 64 = 1024 points per accumulation
+constexpr int TC_WIN = 1024;         // points per accumulation window
 constexpr int TC_TMEM_COLS = TC_TILES * TC_N;   // 512: all of an SM's tensor memory
-// operand layout: core matrix (8 rows x 8 BF16 = 128 B) of slice s, row group g (rows
-// 8g..8g+7, i.e. columns of W), K group kg (points 8kg..8kg+7) at
-// ((s * 8 + g) * 8 + kg) * 128 bytes; LBO (next core matrix along K) = 128 B, SBO (next
-// 8-row group) = 1024 B
-constexpr int TC_LBO = 128;
+// operand layout: K-major with the 128-byte swizzle.  A digit row (one slice of one column of W)
+// holds a stage's 64 points in 128 bytes; its 16-byte chunk g (8 points) sits at chunk
+// g ^ (row % 8), so that the eight chunks of a row, stored by eight neighbouring threads, hit
+// distinct banks; groups of 8 rows are SBO = 1024 bytes apart.  Slices follow one another, so B
+// operands of 2 or 4 slices (N = 128, 256) are one descriptor.  The order of the points within a
+// row is free (the same for all rows): thread g's chunk holds the point pairs g, g + 8, g + 16
+// and g + 24 of the stage, and a warp's loads take whole 128-byte lines.
 constexpr int TC_SBO = 1024;
 constexpr int TC_STAGE_BYTES = TC_SLICES * 8 * TC_SBO;   // 64 KiB
-static_assert(2 * TC_STAGE_BYTES >= TC_N * TC_N * (int)sizeof(double), "the stage buffers hold the half sums");
+constexpr int TC_NS = 2;                                 // stages in the digit ring
+constexpr int TC_SMEM = TC_NS * TC_STAGE_BYTES + 48 * TC_PROD * 4;   // + the exact sums
 constexpr long long TC_SPIN_LIMIT = 1LL << 24;   // polls of an mbarrier (~1 s with the sleeps)
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
     return (unsigned)__cvta_generic_to_shared(p);
 }
 
-// UMMA shared-memory matrix descriptor (K-major, no swizzle): start address, leading
-// (K) and stride (M/N) byte offsets, each >> 4; descriptor version 1 at bit 46.
+// UMMA shared-memory matrix descriptor (K-major, 128-byte swizzle = 2 at bit 61): start address
+// and stride (8-row group) byte offset, each >> 4; descriptor version 1 at bit 46.  A K-step of
+// 16 points advances the start by 32 bytes.
 __device__ __forceinline__ uint64_t umma_desc(unsigned saddr) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(TC_LBO >> 4) << 16) |
-           ((uint64_t)(TC_SBO >> 4) << 32) | (1ull << 46);
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(TC_SBO >> 4) << 32) | (1ull << 46) |
+           (2ull << 61);
 }
 
 // Instruction descriptor of kind::f16: D FP32 (bits 4-5 = 1), A and B BF16 (bits 7-9 and
 // 10-12 = 1), both K-major, N >> 3 at bit 17, M >> 4 at bit 24.
-constexpr unsigned TC_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(TC_N >> 3) << 17) |
-                              ((unsigned)(128 >> 4) << 24);
+constexpr unsigned tc_idesc(int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(n >> 3) << 17) | ((unsigned)(128 >> 4) << 24);
+}
 
+template <int N>
 __device__ __forceinline__ void mma_bf16(unsigned tmem_d, uint64_t adesc, uint64_t bdesc, unsigned accum) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(TC_IDESC), "r"(accum));
+        "l"(adesc), "l"(bdesc), "r"(tc_idesc(N)), "r"(accum));
 }
 
 __device__ __forceinline__ void mma_commit(unsigned mbar) {
@@ -110,20 +118,6 @@ __device__ __forceinline__ bool mbar_wait(unsigned mbar, unsigned parity, long l
     return false;
 }
 
-__device__ __forceinline__ void tmem_ld16(unsigned taddr, float (&v)[16]) {
-    unsigned r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
-        "%13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-          "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int e = 0; e < 16; ++e) v[e] = __uint_as_float(r[e]);
-}
-
 __device__ __forceinline__ void tmem_ld8(unsigned taddr, float (&v)[8]) {
     unsigned r[8];
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
@@ -132,32 +126,6 @@ __device__ __forceinline__ void tmem_ld8(unsigned taddr, float (&v)[8]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(r[e]);
-}
-
-// Fixed-point value of x in units of 2^(e - 56) (|x| < 2^(e - 2), so |result| < 2^54),
-// truncated toward zero, from the bits of x (integer operations only).
-__device__ __forceinline__ long long fixed56(double x, int e) {
-    const long long bits = __double_as_longlong(x);
-    const int ex = (int)((bits >> 52) & 0x7FF);
-    if (ex == 0) return 0;   // zero or subnormal (below 2^-1022)
-    const long long mant = (bits & 0xFFFFFFFFFFFFFll) | 0x10000000000000ll;
-    const int sh = ex - 1019 - e;   // x * 2^(56 - e) = mant * 2^sh, sh <= 1
-    long long y;
-    if (sh >= 0) y = mant << sh;
-    else y = (sh <= -63) ? 0 : (mant >> (-sh));
-    return bits < 0 ? -y : y;
-}
-
-// Balanced base-128 digits of y (|y| < 2^54): y = sum_{s=1..8} d_s 128^(8-s),
-// d_s in [-64, 63].  The low 28 bits of y give the four lower digits (and a carry of 0 or
-// 1 into the high part), the high part the four upper ones, all in 32-bit integers.  (The
-// seven lower steps leave |y| < 2^54 / 128^7 + 1/2 < 33, so the top digit takes what is
-// left without a carry.)  The kernel runs these steps for 8 values in lockstep.
-
-// two small integers (|a|, |b| <= 64, exact in BF16) as a packed BF16 pair, a in the low half
-__device__ __forceinline__ unsigned pack_bf16x2(int a, int b) {
-    const __nv_bfloat162 p = __floats2bfloat162_rn((float)a, (float)b);
-    return *reinterpret_cast<const unsigned*>(&p);
 }
 
 }  // namespace
@@ -218,276 +186,6 @@ __global__ void __launch_bounds__(256) colmax_kernel(GramArgs a, long long CH, u
         unsigned long long t = 0ull;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t = umax64(t, red[w][threadIdx.x]);
         if (t) atomicMax(colmax + (size_t)b * ld + threadIdx.x, t);
-    }
-}
-
-__global__ void __launch_bounds__(TC_THREADS, 1) gram_tc_kernel(GramArgs a, long long CH, int chunks,
-                                                                const unsigned long long* colmax, int ld,
-                                                                int* err, long long limit) {
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ __align__(8) unsigned long long s_mbar[2];
-    __shared__ unsigned s_tmem;
-    __shared__ int s_e[TC_N];
-    __shared__ int s_last;
-    unsigned char* stages = smem_raw;   // two stages of TC_STAGE_BYTES, 1024-aligned
-    double* sacc = reinterpret_cast<double*>(smem_raw);   // reused for the bottom-half sums
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const unsigned mbar0 = smem_u32(&s_mbar[0]);
-    const unsigned stage_s = smem_u32(stages);
-
-    if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar0) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar0 + 8) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
-                     "r"(TC_TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const unsigned tmem = s_tmem;
-    unsigned parity[2] = {0u, 0u};
-    bool pending[2] = {false, false};   // a commit on this stage buffer not yet waited for
-    bool failed = false;
-    // wait for the MMAs that read stage buffer q (all threads; one vote decides)
-    auto wait_buf = [&](int q) -> bool {
-        if (!pending[q]) return true;
-        const bool ok = mbar_wait(mbar0 + 8u * q, parity[q], limit);
-        parity[q] ^= 1u;
-        pending[q] = false;
-        return __syncthreads_or(ok ? 0 : 1) == 0;
-    };
-    // drain rows: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (its lane = accumulator
-    // row r) and the 32 columns 32 (w / 4) .. + 31; rows r < 64 hold the products with
-    // s + t = c (top), rows r >= 64 those with s + t = c + 1 (bottom)
-    const int row = 32 * (warp & 3) + lane;
-    const int cbase = 32 * (warp >> 2);
-    const bool top = row < 64;
-    const int irow = top ? row : row - 64;
-    // tiles c0 = 0..3 and 4..7 fold into exact 46-bit integers H, Lo (weights 2^(7(3-c0)),
-    // 2^(7(7-c0))), worth H 2^(-7(5+d)) + Lo 2^(-7(9+d)) with d = 0 (top) or 1 (bottom)
-    const double wH = ldexp(1.0, -7 * (5 + (top ? 0 : 1)));
-    const double wL = ldexp(1.0, -7 * (9 + (top ? 0 : 1)));
-    double acc[32];
-    int prevK = TC_N;   // rows [K, prevK) of the stage buffers may hold another item's digits
-
-    const int units = a.B * chunks;
-    for (int u = blockIdx.x; u < units && !failed; u += gridDim.x) {
-        const int b = u / chunks, chunk = u - b * chunks;
-        const int K = a.KA[b];
-        const long long p_lo = (long long)chunk * CH, p_hi = min(a.Ng, p_lo + CH);
-        const void* const* cols = a.colsA + (size_t)b * a.ldcols;
-        if (tid < TC_N) {
-            const unsigned long long m = (tid < K) ? colmax[(size_t)b * ld + tid] : 0ull;
-            // 2^(e - 2) > max |W[:, i]|:  e = unbiased exponent of the maximum + 3
-            s_e[tid] = m ? (int)((m >> 52) & 0x7FF) - 1023 + 3 : 0;
-        }
-        if (K < prevK) {   // zero the digit rows of columns K .. prevK - 1 in both buffers
-            const int nrow = prevK - K;
-            for (int e = tid; e < 2 * TC_SLICES * nrow * 8; e += TC_THREADS) {
-                const int bufq = e / (TC_SLICES * nrow * 8);
-                const int r = e - bufq * TC_SLICES * nrow * 8;
-                const int sl = r / (nrow * 8), rest = r - sl * nrow * 8;
-                const int col = K + rest / 8, kg = rest & 7;
-                *reinterpret_cast<uint4*>(stages + bufq * TC_STAGE_BYTES +
-                                          ((sl * 8 + (col >> 3)) * 8 + kg) * 128 + (col & 7) * 16) =
-                    make_uint4(0u, 0u, 0u, 0u);
-            }
-        }
-        prevK = K;
-#pragma unroll
-        for (int j = 0; j < 32; ++j) acc[j] = 0.0;
-        __syncthreads();
-        int nst = 0, si = 0;   // stages since the last drain; stage counter of the unit
-        for (long long p0 = p_lo; p0 < p_hi; p0 += TC_PTS, ++si) {
-            const int q = si & 1;
-            unsigned char* stage = stages + q * TC_STAGE_BYTES;
-            // ---- this thread's items of the stage (one column and 8 consecutive points
-            //      each; item it -> row rho = it & 7 of row group it >> 6, K group
-            //      (it >> 3) & 7, so that 8 consecutive threads fill one 128-byte core-
-            //      matrix row): all their loads are issued before anything waits
-            double xr[2][8];
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const int it = tid + r * TC_THREADS;
-                const int col = ((it >> 6) << 3) | (it & 7), kg = (it >> 3) & 7;
-                const long long pb = p0 + kg * 8;
-#pragma unroll
-                for (int k = 0; k < 8; ++k) xr[r][k] = 0.0;
-                if (col < K) {
-                    const double* c = reinterpret_cast<const double*>(cols[col]);
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        if (pb + k < p_hi) xr[r][k] = c[pb + k];
-                }
-            }
-            if (!wait_buf(q)) {   // the MMAs that read this buffer two stages ago
-                failed = true;
-                break;
-            }
-            // ---- digits into the stage buffer (columns >= K stay zero): the 8 points of an
-            //      item are cut in lockstep, digit by digit (8 independent chains), and each
-            //      slice's 16-byte core-matrix row is stored as soon as it is complete
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const int it = tid + r * TC_THREADS;
-                const int col = ((it >> 6) << 3) | (it & 7), kg = (it >> 3) & 7;
-                if (col >= K) continue;
-                const int e = s_e[col];
-                int lo[8], hi[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const long long y = fixed56(xr[r][k], e);
-                    lo[k] = (int)(y & 0xFFFFFFFll);
-                    hi[k] = (int)(y >> 28);
-                }
-                unsigned char* rowp = stage + ((col >> 3) * 8 + kg) * 128 + (col & 7) * 16;
-#pragma unroll
-                for (int sl = TC_SLICES - 1; sl >= 0; --sl) {
-                    int d[8];
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        int& v = (sl >= TC_SLICES / 2) ? lo[k] : hi[k];
-                        d[k] = ((v + 64) & 127) - 64;
-                        v = (v - d[k]) >> 7;
-                        if (sl == TC_SLICES / 2) hi[k] += lo[k];   // the carry out of the low half
-                    }
-                    *reinterpret_cast<uint4*>(rowp + sl * 8 * TC_SBO) =
-                        make_uint4(pack_bf16x2(d[0], d[1]), pack_bf16x2(d[2], d[3]), pack_bf16x2(d[4], d[5]),
-                                   pack_bf16x2(d[6], d[7]));
-                }
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncthreads();
-            // ---- 4 K-steps of 16 points x 20 (s, t) pairs, committed to this buffer's mbarrier
-            if (tid == 0) {
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const unsigned sb = stage_s + q * TC_STAGE_BYTES;
-                const unsigned first = (nst == 0) ? 0u : 1u;   // 0: the window's first write of a tile
-#pragma unroll
-                for (int k = 0; k < TC_PTS / 16; ++k) {
-#pragma unroll
-                    for (int sa = 0; sa < TC_SLICES; sa += 2) {   // A: slices sa, sa + 1 (0-based)
-#pragma unroll
-                        for (int t = 0; t < TC_TILES; ++t) {      // B: slice t; tile c0 = sa + t
-                            if (sa + t >= TC_TILES) continue;
-                            const int c0 = sa + t;
-                            // the first pair into tile c0 in issue order is (sa = 0, t = c0) for
-                            // c0 < 8; it overwrites the tile at the window's first K-step
-                            const unsigned acc = (k == 0 && sa == 0) ? first : 1u;
-                            mma_bf16(tmem + (unsigned)(c0 * TC_N),
-                                     umma_desc(sb + (sa * 8) * TC_SBO + (2 * k) * TC_LBO),
-                                     umma_desc(sb + (t * 8) * TC_SBO + (2 * k) * TC_LBO), acc);
-                        }
-                    }
-                }
-                mma_commit(mbar0 + 8u * q);
-            }
-            pending[q] = true;
-            ++nst;
-            if (nst == TC_STAGES_PER_DRAIN || p0 + TC_PTS >= p_hi) {
-                // ---- drain: every MMA so far has completed once both buffers are waited for
-                if (!wait_buf(q) || !wait_buf(q ^ 1)) {
-                    failed = true;
-                    break;
-                }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const unsigned lane_base = tmem + ((unsigned)(32 * (warp & 3)) << 16) + (unsigned)cbase;
-#pragma unroll
-                for (int j0 = 0; j0 < 32; j0 += 16) {
-                    long long H[16], Lo[16];
-#pragma unroll
-                    for (int e2 = 0; e2 < 16; ++e2) H[e2] = Lo[e2] = 0ll;
-#pragma unroll
-                    for (int c0 = 0; c0 < TC_TILES; ++c0) {
-                        float v[16];
-                        tmem_ld16(lane_base + (unsigned)(c0 * TC_N + j0), v);
-#pragma unroll
-                        for (int e2 = 0; e2 < 16; ++e2) {
-                            const long long x = (long long)__float2int_rn(v[e2]);   // an exact integer
-                            if (c0 < 4) H[e2] += x << (7 * (3 - c0));
-                            else Lo[e2] += x << (7 * (7 - c0));
-                        }
-                    }
-#pragma unroll
-                    for (int e2 = 0; e2 < 16; ++e2)
-                        acc[j0 + e2] = fma((double)H[e2], wH, fma((double)Lo[e2], wL, acc[j0 + e2]));
-                }
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                __syncthreads();
-                nst = 0;
-            }
-        }
-        if (failed) break;
-        // ---- the unit's partial Gram: top + bottom halves, scaled by 2^(e_i + e_j)
-        __syncthreads();   // every MMA of the unit completed (drained): the buffers are free
-        if (!top) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) sacc[irow * TC_N + cbase + j] = acc[j];
-        }
-        __syncthreads();
-        const size_t outsz = (size_t)a.maxKA * a.maxKB;
-        double* mypart = a.part + ((size_t)b * chunks + chunk) * outsz;
-        if (top && irow < K) {
-            const int ei = s_e[irow];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const int jj = cbase + j;
-                if (jj >= irow && jj < K)
-                    mypart[(size_t)irow * a.maxKB + jj] = ldexp(acc[j] + sacc[irow * TC_N + jj], ei + s_e[jj]);
-            }
-        }
-        // the last unit of item b sums the chunk partials in chunk order
-        __threadfence();
-        __syncthreads();
-        if (tid == 0) {
-            const unsigned ticket = atom_add_acq_rel_u32(a.counter + b, 1u);
-            s_last = (ticket == (unsigned)chunks - 1u);
-        }
-        __syncthreads();
-        if (s_last) {
-            __threadfence();
-            const double* bpart = a.part + (size_t)b * chunks * outsz;
-            double* Gb = a.G + (size_t)b * a.ldG_b;
-            for (int o = tid; o < K * K; o += TC_THREADS) {
-                const int i = o / K, j = o - i * K;
-                if (j < i) continue;
-                // chunk order (reproducible), loads in batches of 16 independent ones
-                const double* src = bpart + (size_t)i * a.maxKB + j;
-                double sum = 0.0;
-                int cc = 0;
-                for (; cc + 16 <= chunks; cc += 16) {
-                    double v[16];
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) v[e] = src[(size_t)(cc + e) * outsz];
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) sum += v[e];
-                }
-                for (; cc < chunks; ++cc) sum += src[(size_t)cc * outsz];
-                Gb[(size_t)i * a.ldG + j] = sum;
-                Gb[(size_t)j * a.ldG + i] = sum;
-            }
-            if (tid == 0) st_relaxed_u32(a.counter + b, 0u);
-        }
-        __syncthreads();
-    }
-    if (failed) {
-        if (tid == 0) record_error(err, DERR_TIMEOUT);
-        // MMAs may still be running: wait once more (bounded) on both buffers before the
-        // tensor memory is released
-        for (int q = 0; q < 2; ++q)
-            if (pending[q]) mbar_wait(mbar0 + 8u * q, parity[q]);
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (warp == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_TMEM_COLS)
-                     : "memory");
     }
 }
 
@@ -719,7 +417,7 @@ __global__ void __launch_bounds__(N2_THREADS, 1) gram_tc32_kernel(GramArgs a, lo
                             const unsigned sb = stage_s + q * N2_STAGE_BYTES;
 #pragma unroll
                             for (int k = 0; k < N2_PTS / 16; ++k)
-                                mma_n256(td, umma_desc(sb + k * 2 * TC_LBO), (p0 == w0 && k == 0) ? 0u : 1u);
+                                mma_n256(td, umma_desc(sb + k * 32), (p0 == w0 && k == 0) ? 0u : 1u);
                         }
                         mma_commit(empty0 + 8u * q);
                     }
@@ -732,7 +430,7 @@ __global__ void __launch_bounds__(N2_THREADS, 1) gram_tc32_kernel(GramArgs a, lo
         __syncwarp();
     } else {
         // ---------------- producers / read-back (warps 0-7) ----------------
-        const int col = ((tid >> 6) << 3) | (tid & 7), kg = (tid >> 3) & 7;
+        const int col = tid >> 3, g8 = tid & 7;   // this thread's column and chunk of a stage
         const int qd = warp & 3, ch = warp >> 2;   // read-back: lane quarter (slice s) and column half
         bool bad = false;
         int gw = 0;
@@ -762,29 +460,29 @@ __global__ void __launch_bounds__(N2_THREADS, 1) gram_tc32_kernel(GramArgs a, lo
             P.p0 += N2_PTS;
             if (P.p0 >= P.hi) set_unit(P, P.u + gridDim.x);
         };
-        // this thread's 8 values of a stage (column col, points kg * 8 ..), copied by cp.async
-        // into its own 16-byte chunks of a staging slot: chunk k (points 2k, 2k + 1) at
-        // (k * 256 + tid) * 16, so that a warp's reads hit distinct banks; points past the
+        // this thread's 8 values of a stage, copied by cp.async into its own 16-byte chunks of a
+        // staging slot: chunk k (the point pair g8 + 8 k) at (k * 256 + tid) * 16, so that a warp's reads hit distinct banks; points past the
         // unit are zero-filled (source size 0 reads nothing).  Columns >= K are neither
         // copied nor cut: their digit rows reach no output that is read back.
         const unsigned stg_s = smem_u32(stg) + (unsigned)tid * 16u;
         auto issue = [&](const Pos& P, int slot) {
             if (P.c == nullptr) return;
-            const long long pb = P.p0 + kg * 8;
+            const long long pb = P.p0 + 2 * g8;
             const unsigned d0 = stg_s + (unsigned)(slot * N2_STG_BYTES);
-            if (pb + 8 <= P.hi && ((reinterpret_cast<uintptr_t>(P.c) & 15u) == 0)) {
+            if (P.p0 + N2_PTS <= P.hi && ((reinterpret_cast<uintptr_t>(P.c) & 15u) == 0)) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d0 + (unsigned)(k * 256 * 16)),
-                                 "l"(P.c + pb + 2 * k)
+                                 "l"(P.c + pb + 16 * k)
                                  : "memory");
                 return;
             }
 #pragma unroll
             for (int k = 0; k < 8; ++k) {   // 8-byte copies (ragged tail or 8-byte aligned columns)
-                const bool v = pb + k < P.hi;
+                const long long pk = pb + 16 * (k >> 1) + (k & 1);
+                const bool v = pk < P.hi;
                 asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d0 + (unsigned)((k >> 1) * 256 * 16 + (k & 1) * 8)),
-                             "l"(v ? P.c + pb + k : P.c), "r"(v ? 8u : 0u)
+                             "l"(v ? P.c + pk : P.c), "r"(v ? 8u : 0u)
                              : "memory");
             }
         };
@@ -913,8 +611,8 @@ __global__ void __launch_bounds__(N2_THREADS, 1) gram_tc32_kernel(GramArgs a, lo
                 unsigned zl[8], zh[8];
 #pragma unroll
                 for (int k = 0; k < 8; ++k) cut56(xc[k], ce, zl[k], zh[k]);
-                // slice s holds digit k = 7 - s (bits 7k .. 7k + 6 of z); row 32 s + col, K group kg
-                unsigned char* rowp = smem_raw + q * N2_STAGE_BYTES + ((col >> 3) * 8 + kg) * 128 + (col & 7) * 16;
+                // slice s holds digit k = 7 - s (bits 7k .. 7k + 6 of z); row 32 s + col
+                unsigned char* rowp = smem_raw + q * N2_STAGE_BYTES + col * 128 + ((g8 ^ (col & 7)) << 4);
 #define N2_SLICE(S)                                                                                        \
     *reinterpret_cast<uint4*>(rowp + (S) * 4 * 1024) =                                                     \
         make_uint4(digit_pair<7 * (7 - (S))>(zl[0], zh[0], zl[1], zh[1]),                                  \
@@ -956,6 +654,311 @@ __global__ void __launch_bounds__(N2_THREADS, 1) gram_tc32_kernel(GramArgs a, lo
     }
 }
 
+// ---------------------------------------------------------------------------------------
+// Wide form, K <= 64 columns (see the head of this file).
+
+namespace {
+
+// four columns of two accumulator tiles
+__device__ __forceinline__ void tmem_ld4(unsigned taddr, int (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr));
+}
+
+__device__ __forceinline__ void tc_prod_sync() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
+
+// (w0, w1, w2) += the 96-bit integer H 2^28 + L
+__device__ __forceinline__ void add96(unsigned (&w)[3], long long H, long long L) {
+    const unsigned long long h = (unsigned long long)H << 28;
+    const unsigned h2 = (unsigned)(int)(H >> 36), l2 = (unsigned)(int)(L >> 63);
+    asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+        : "+r"(w[0]), "+r"(w[1]), "+r"(w[2])
+        : "r"((unsigned)h), "r"((unsigned)(h >> 32)), "r"(h2));
+    asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+        : "+r"(w[0]), "+r"(w[1]), "+r"(w[2])
+        : "r"((unsigned)L), "r"((unsigned)((unsigned long long)L >> 32)), "r"(l2));
+}
+
+}  // namespace
+
+// 17 warps: five share one SM sub-partition's 16K registers, so at most 96 a thread (the bound of
+// 640 threads says so); the exact sums, touched once a window, live in shared memory
+__global__ void __launch_bounds__(640, 1) gram_tc_kernel(GramArgs a, int CH, int chunks,
+                                                                const unsigned long long* colmax, int ld,
+                                                                int* err, long long limit) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    __shared__ __align__(8) unsigned long long s_bar[2 * TC_NS + 3];
+    __shared__ unsigned s_tmem;
+    __shared__ volatile int s_fail;
+    __shared__ int s_last;
+    unsigned* sv = reinterpret_cast<unsigned*>(smem_raw + TC_NS * TC_STAGE_BYTES);   // [16 x 3][TC_PROD]
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const unsigned full0 = smem_u32(&s_bar[0]);          // [TC_NS], TC_PROD arrivals
+    const unsigned empty0 = smem_u32(&s_bar[TC_NS]);     // [TC_NS], MMA commit
+    const unsigned tfull = smem_u32(&s_bar[2 * TC_NS]);  // MMA commit of a window
+    const unsigned tempty = tfull + 8;                   // TC_PROD arrivals: a window is read back
+    const unsigned done = tfull + 16;                    // MMA commit at exit
+    const unsigned stage_s = smem_u32(smem_raw);
+    if (tid == 0) {
+        for (int q = 0; q < TC_NS; ++q) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(full0 + 8u * q), "r"(TC_PROD) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(empty0 + 8u * q) : "memory");
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tfull) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(tempty), "r"(TC_PROD) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(done) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_fail = 0;
+    }
+    // zero the ring once (digit rows of columns >= K then only ever hold digits of earlier
+    // items, which reach no output read back)
+    for (int e = tid; e < TC_NS * TC_STAGE_BYTES / 16; e += TC_THREADS)
+        reinterpret_cast<uint4*>(smem_raw)[e] = make_uint4(0u, 0u, 0u, 0u);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (warp == 16) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                     "r"(TC_TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const unsigned tmem = s_tmem;
+    const int Ng = (int)a.Ng, units = a.B * chunks;
+
+    if (warp == 16) {
+        // ---------------- MMA issue (one thread) ----------------
+        if (lane == 0) {
+            int gs = 0, gw = 0;
+            bool bad = false;
+            for (int u = blockIdx.x; u < units; u += gridDim.x) {
+                const int len = min(Ng - (u % chunks) * CH, CH);
+                for (int rel = 0; rel < len; rel += TC_PTS, ++gs) {
+                    const bool first = rel % TC_WIN == 0;
+                    if (first && !bad && !mbar_wait_f(tempty, (gw & 1) ^ 1, &s_fail, limit)) bad = true;
+                    const int q = gs % TC_NS;
+                    if (!bad && !mbar_wait_f(full0 + 8u * q, (gs / TC_NS) & 1, &s_fail, limit)) bad = true;
+                    if (!bad) {
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+                        for (int k = 0; k < TC_PTS / 16; ++k) {
+                            // slices sa, sa + 1 (A) times slices t .. (B) into the tiles from sa + t; the
+                            // pairs of slices 0, 1 reach every tile and overwrite it at a window's start
+                            const uint64_t d0 = umma_desc(stage_s + q * TC_STAGE_BYTES + 32 * k);
+                            const uint64_t sl = (8 * TC_SBO) >> 4;   // next slice, in descriptor units
+                            const unsigned acc = (k == 0 && first) ? 0u : 1u;
+                            mma_bf16<256>(tmem, d0, d0, acc);
+                            mma_bf16<256>(tmem + 4 * TC_N, d0, d0 + 4 * sl, acc);
+                            mma_bf16<256>(tmem + 2 * TC_N, d0 + 2 * sl, d0, 1u);
+                            mma_bf16<128>(tmem + 6 * TC_N, d0 + 2 * sl, d0 + 4 * sl, 1u);
+                            mma_bf16<256>(tmem + 4 * TC_N, d0 + 4 * sl, d0, 1u);
+                            mma_bf16<128>(tmem + 6 * TC_N, d0 + 6 * sl, d0, 1u);
+                        }
+                    }
+                    mma_commit(empty0 + 8u * q);
+                    if ((rel + TC_PTS) % TC_WIN == 0 || rel + TC_PTS >= len) {
+                        mma_commit(tfull);
+                        ++gw;
+                    }
+                }
+            }
+            mma_commit(done);
+            mbar_wait(done, 0);   // every MMA of this CTA has completed (bounded; also after a failure)
+        }
+        __syncwarp();
+    } else {
+    // ---------------- producers / read-back (warps 0-15) ----------------
+    const int col = tid >> 3, g8 = tid & 7;   // this thread's column and chunk of a stage
+    // read-back: lane quarter warp % 4, columns 16 (warp / 4) .. + 15; accumulator rows r < 64
+    // hold the products with s + t = c (top), rows r >= 64 those with s + t = c + 1 (bottom)
+    const int irow = (32 * (warp & 3) + lane) & 63, cq = warp >> 2;
+    const bool top = (warp & 3) < 2;
+    bool bad = false;
+
+    // the stage whose values are in flight: unit u, points p0 .. of lo .. hi, this thread's column
+    int u = blockIdx.x, hi = 0, p0 = 0, lo = 0;
+    const double* c = nullptr;
+    auto set_unit = [&]() {
+        if (u >= units) return;
+        const int b = u / chunks;
+        lo = p0 = (u - b * chunks) * CH;
+        hi = min(Ng, lo + CH);
+        c = col < a.KA[b] ? reinterpret_cast<const double*>(a.colsA[(size_t)b * a.ldcols + col]) : nullptr;
+    };
+    double x[8];
+    auto load = [&]() {   // columns >= K are neither read nor cut
+        if (u >= units || c == nullptr) return;
+        const int pb = p0 + 2 * g8;
+        if (p0 + TC_PTS <= hi && ((reinterpret_cast<uintptr_t>(c) & 15u) == 0)) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const double2 v = *reinterpret_cast<const double2*>(c + pb + 16 * k);
+                x[2 * k] = v.x;
+                x[2 * k + 1] = v.y;
+            }
+            return;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            x[2 * k] = pb + 16 * k < hi ? c[pb + 16 * k] : 0.0;
+            x[2 * k + 1] = pb + 16 * k + 1 < hi ? c[pb + 16 * k + 1] : 0.0;
+        }
+    };
+    // this thread's 16 outputs: exact 96-bit sums over the unit's windows, word w of output j at
+    // sv[(3 j + w) TC_PROD + tid]
+    int pu = -1, gw = 0;   // unit of the window to read back, windows read back so far
+    bool pfirst = false, plast = false;
+    auto readback = [&]() {
+        if (!bad && !mbar_wait_f(tfull, gw & 1, &s_fail, limit)) bad = true;
+        ++gw;
+        __syncwarp();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const unsigned base = tmem + ((unsigned)(32 * (warp & 3)) << 16) + (unsigned)(16 * cq);
+#pragma unroll
+        for (int j0 = 0; j0 < 16; j0 += 4) {
+            int v[TC_TILES][4];
+#pragma unroll
+            for (int t = 0; t < TC_TILES; ++t) tmem_ld4(base + (unsigned)(t * TC_N + j0), v[t]);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                long long h[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    h[t] = (long long)__float2int_rn(__int_as_float(v[2 * t][e])) * 128 +
+                           __float2int_rn(__int_as_float(v[2 * t + 1][e]));   // exact integers
+                unsigned* v3 = sv + 3 * (j0 + e) * TC_PROD + tid;
+                unsigned w[3] = {0u, 0u, 0u};
+                if (!pfirst) {
+#pragma unroll
+                    for (int t = 0; t < 3; ++t) w[t] = v3[t * TC_PROD];
+                }
+                add96(w, (h[0] << 14) + h[1], (h[2] << 14) + h[3]);
+#pragma unroll
+                for (int t = 0; t < 3; ++t) v3[t * TC_PROD] = w[t];
+            }
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        mbar_arrive(tempty);   // the tiles may be overwritten
+        if (!plast) return;
+        // ---- the unit's partial: 2^7 top + bottom (64 rows, two warps on), rounded once
+        tc_prod_sync();
+        const int b = pu / chunks, chunk = pu - b * chunks;
+        const int K = a.KA[b];
+        const size_t outsz = (size_t)a.maxKA * a.maxKB;
+        double* mypart = a.part + ((size_t)b * chunks + chunk) * outsz;
+        if (top && irow < K) {
+            const int ei = col_exp(colmax[(size_t)b * ld + irow]);
+#pragma unroll 1
+            for (int j = 0; j < 16; ++j) {
+                const int jj = 16 * cq + j;
+                if (jj < irow || jj >= K) continue;
+                const unsigned* v = sv + 3 * j * TC_PROD + tid;
+                auto word = [&](int o) {
+                    return ((__int128)(int)v[2 * TC_PROD + o] << 64) |
+                           ((unsigned long long)v[TC_PROD + o] << 32 | v[o]);
+                };
+                mypart[(size_t)irow * a.maxKB + jj] =
+                    i128_to_double((word(0) << 7) + word(64), ei + col_exp(colmax[(size_t)b * ld + jj]) - 70);
+            }
+        }
+        // the last unit of item b sums the chunk partials in chunk order
+        __threadfence();
+        tc_prod_sync();
+        if (tid == 0) {
+            const unsigned ticket = atom_add_acq_rel_u32(a.counter + b, 1u);
+            s_last = (ticket == (unsigned)chunks - 1u);
+        }
+        tc_prod_sync();
+        if (s_last) {
+            __threadfence();
+            const double* bpart = a.part + (size_t)b * chunks * outsz;
+            double* Gb = a.G + (size_t)b * a.ldG_b;
+            for (int o = tid; o < K * K; o += TC_PROD) {
+                const int i = o / K, j = o - i * K;
+                if (j < i) continue;
+                // chunk order (reproducible), loads in batches of 8 independent ones
+                const double* src = bpart + (size_t)i * a.maxKB + j;
+                double sum = 0.0;
+                int cc = 0;
+                for (; cc + 8 <= chunks; cc += 8) {
+                    double v[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) v[e] = src[(size_t)(cc + e) * outsz];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) sum += v[e];
+                }
+                for (; cc < chunks; ++cc) sum += src[(size_t)cc * outsz];
+                Gb[(size_t)i * a.ldG + j] = sum;
+                Gb[(size_t)j * a.ldG + i] = sum;
+            }
+            if (tid == 0) st_relaxed_u32(a.counter + b, 0u);
+        }
+        tc_prod_sync();
+    };
+
+    set_unit();
+    load();
+    int gs = 0, ce = 0;
+    while (u < units) {
+        const int q = gs % TC_NS;
+        const bool mine = c != nullptr;
+        const int cu = u, rel = p0 - lo, len = hi - lo;   // the stage at hand
+        if (rel == 0) ce = col_exp(mine ? colmax[(size_t)(u / chunks) * ld + col] : 0ull) + 1020;
+        unsigned zl[8], zh[8];
+        if (mine) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) cut56(x[k], ce, zl[k], zh[k]);
+        }
+        // the next stage's values travel while this one's digits are stored
+        p0 += TC_PTS;
+        if (p0 >= hi) {
+            u += gridDim.x;
+            set_unit();
+        }
+        load();
+        if (!bad && !mbar_wait_f(empty0 + 8u * q, ((gs / TC_NS) & 1) ^ 1, &s_fail, limit)) bad = true;
+        if (mine) {
+            unsigned char* rowp = smem_raw + q * TC_STAGE_BYTES + col * 128 + ((g8 ^ (col & 7)) << 4);
+#define TC_SLICE(S)                                                                                        \
+    *reinterpret_cast<uint4*>(rowp + (S) * 8 * TC_SBO) =                                                   \
+        make_uint4(digit_pair<7 * (7 - (S))>(zl[0], zh[0], zl[1], zh[1]),                                  \
+                   digit_pair<7 * (7 - (S))>(zl[2], zh[2], zl[3], zh[3]),                                  \
+                   digit_pair<7 * (7 - (S))>(zl[4], zh[4], zl[5], zh[5]),                                  \
+                   digit_pair<7 * (7 - (S))>(zl[6], zh[6], zl[7], zh[7]));
+            TC_SLICE(0) TC_SLICE(1) TC_SLICE(2) TC_SLICE(3) TC_SLICE(4) TC_SLICE(5) TC_SLICE(6) TC_SLICE(7)
+#undef TC_SLICE
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        }
+        mbar_arrive(full0 + 8u * q);
+        ++gs;
+        // A finished window is read back a stage later, which waits in the ring meanwhile (one
+        // set of tiles fills the tensor memory).
+        const bool wlast = (rel + TC_PTS) % TC_WIN == 0 || rel + TC_PTS >= len;
+        if (pu >= 0) {
+            readback();
+            pu = -1;
+        }
+        if (wlast) {
+            pu = cu;
+            pfirst = rel < TC_WIN;
+            plast = rel + TC_PTS >= len;
+        }
+    }
+    if (pu >= 0) readback();
+    }
+    if (s_fail && tid == 0) record_error(err, DERR_TIMEOUT);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 16) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_TMEM_COLS)
+                     : "memory");
+    }
+}
+
 int gram_tc_max_cols() { return TC_N; }
 
 cudaError_t launch_gram_tc(const GramArgs& a, unsigned long long* colmax, int ld, int* err, long long spin_limit,
@@ -975,11 +978,6 @@ cudaError_t launch_gram_tc(const GramArgs& a, unsigned long long* colmax, int ld
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // one CTA an SM: the tiles take all 512 tensor-memory columns, and the two stage
-    // buffers (128 KiB of shared memory) keep a second CTA off the SM
-    const size_t smem = 2 * TC_STAGE_BYTES;
-    e = cudaFuncSetAttribute((const void*)gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     if (a.maxKA <= N2_COLS && chunks >= 2) {
         // narrow form: units of U points (at least two per partial slot of the other Gram
         // kernels, since a unit's partial is K x K 128-bit integers)
@@ -994,8 +992,17 @@ cudaError_t launch_gram_tc(const GramArgs& a, unsigned long long* colmax, int ld
         ++g_launch_count;
         return cudaGetLastError();
     }
-    const int grid = std::max(1, std::min(sms, a.B * chunks));
-    gram_tc_kernel<<<grid, TC_THREADS, smem, st>>>(a, CH, chunks, colmax, ld, err, spin_limit);
+    // wide form, one CTA an SM (the tiles take all 512 tensor-memory columns, the ring most of the
+    // shared memory): chunks that fill whole waves of the grid where there are several waves
+    // (4 windows of 128^3: 512 units of 16384 points were 3.4 waves of 152)
+    const int waves = std::max(1, a.B * chunks / std::max(1, sms));
+    const int cw = std::min(chunks, std::max(1, (int)((long long)waves * sms / a.B)));
+    const int CHw = (int)(((a.Ng + cw - 1) / cw + TC_PTS - 1) / TC_PTS * TC_PTS);
+    const int chunksw = (int)((a.Ng + CHw - 1) / CHw);
+    e = cudaFuncSetAttribute((const void*)gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+    if (e != cudaSuccess) return e;
+    const int grid = std::max(1, std::min(sms, a.B * chunksw));
+    gram_tc_kernel<<<grid, TC_THREADS, TC_SMEM, st>>>(a, CHw, chunksw, colmax, ld, err, spin_limit);
     ++g_launch_count;
     return cudaGetLastError();
 }
