@@ -529,29 +529,40 @@ __global__ void __launch_bounds__(256) tsmm_kernel(TsmmArgs a) {
     }
 }
 
-// Out_b = In_b C_b with FP64 input and output in double-float arithmetic (FP32 mode):
-// one thread per point, blocks of J <= 16 outputs.  C sits in shared memory as float-pair
-// planes hi, lo (rows padded to a multiple of 4, read as warp-wide broadcasts); each input
-// is split once per block (d2df_bits) and broadcast into both lanes of a packed pair, so
-// one df_mac2 serves two outputs.  The inputs travel by cp.async in groups of TSMM_TG into
-// the thread's own shared-memory slots, one group ahead (no registers held, no barrier:
+// Out_b = In_b C_b with FP64 input and output in double-float arithmetic (FP32 mode): P points
+// a thread (256 apart), blocks of J <= 16 outputs, J even.  C sits in shared memory as
+// float-pair planes hi, lo (rows padded to a multiple of 4, read as warp-wide broadcasts);
+// each input is split once per block (d2df_bits) and broadcast into both lanes of a packed
+// pair, so one df_mac2 serves two outputs.  The inputs travel by cp.async in groups of TSMM_TG
+// into the thread's own shared-memory slots, one group ahead (no registers held, no barrier:
 // each thread reads back only its own copies).
-constexpr int TSMM_TG = 8;
-template <int J>
+// Issue slots and the FP32 pipe bound it (126 instructions a point and input with one point a
+// thread and J a multiple of 4, 48 of them packed arithmetic, for 6 outputs): two points share
+// C's loads, the column pointers and the loop, and J follows the outputs by twos.  64
+// windows of 32 snapshots on 64^3, 6 modes: 2.5 -> 2.1 ms.
+constexpr int TSMM_TG = 4;
+template <int J, int P>
 __device__ __forceinline__ void tsmm_df_block(const void* const* cols, int KIN, const float* sC, int pl, int KP,
-                                              int j0, int jn, long long p, long long Ng, double* out,
-                                              double* stg, int nthr) {
-    constexpr int H = J / 2;
-    f2p sh[H], sl[H];
+                                              int j0, int jn, int p, int Ng, double* out, double* stg) {
+    constexpr int H = J / 2, NT = 256;
+    f2p sh[P][H], sl[P][H];
 #pragma unroll
-    for (int h = 0; h < H; ++h) sh[h] = sl[h] = 0ull;
-    // stg: this thread's slots, [slot][k][thread] (thread-contiguous: no bank conflicts)
-    auto slot_of = [&](int sl2, int k) { return stg + (size_t)(sl2 * TSMM_TG + k) * nthr; };
+    for (int t = 0; t < P; ++t)
+#pragma unroll
+        for (int h = 0; h < H; ++h) sh[t][h] = sl[t][h] = 0ull;
+    // stg: this thread's slots, [slot][k][point][thread] (thread-contiguous: no bank conflicts)
+    auto slot_of = [&](int sl2, int k, int t) { return stg + ((sl2 * TSMM_TG + k) * P + t) * NT; };
     auto issue = [&](int g, int sl2) {
 #pragma unroll
         for (int k = 0; k < TSMM_TG; ++k) {
             const int i = g * TSMM_TG + k;
-            if (i < KIN) cp_async8(slot_of(sl2, k), reinterpret_cast<const double*>(cols[i]) + p, 8);
+            if (i >= KIN) break;
+            const double* c = reinterpret_cast<const double*>(cols[i]);
+#pragma unroll
+            for (int t = 0; t < P; ++t) {
+                const bool ok = t == 0 || p + t * NT < Ng;
+                cp_async8(slot_of(sl2, k, t), ok ? c + p + t * NT : c, ok ? 8 : 0);
+            }
         }
         cp_async_commit();
     };
@@ -564,27 +575,48 @@ __device__ __forceinline__ void tsmm_df_block(const void* const* cols, int KIN, 
         for (int k = 0; k < TSMM_TG; ++k) {
             const int i = g * TSMM_TG + k;
             if (i >= KIN) break;
-            const float2 x = d2df_bits(*slot_of(g & 1, k));
-            const f2p xh = pk2(x.x, x.x), nxh = pk2(-x.x, -x.x), xl = pk2(x.y, x.y);
-            const float* row = sC + (size_t)i * KP + j0;
+            f2p xh[P], nxh[P], xl[P];
 #pragma unroll
-            for (int h4 = 0; h4 < J / 4; ++h4) {
-                const ulonglong2 ch = *reinterpret_cast<const ulonglong2*>(row + 4 * h4);
-                const ulonglong2 cl = *reinterpret_cast<const ulonglong2*>(row + pl + 4 * h4);
-                df_mac2(sh[2 * h4], sl[2 * h4], xh, nxh, xl, ch.x, cl.x);
-                df_mac2(sh[2 * h4 + 1], sl[2 * h4 + 1], xh, nxh, xl, ch.y, cl.y);
+            for (int t = 0; t < P; ++t) {
+                const float2 x = d2df_bits(*slot_of(g & 1, k, t));
+                xh[t] = pk2(x.x, x.x);
+                nxh[t] = pk2(-x.x, -x.x);
+                xl[t] = pk2(x.y, x.y);
+            }
+            const float* row = sC + i * KP + j0;
+#pragma unroll
+            for (int h = 0; h < H; h += 2) {
+                ulonglong2 ch, cl;
+                if (h + 1 < H) {
+                    ch = *reinterpret_cast<const ulonglong2*>(row + 2 * h);
+                    cl = *reinterpret_cast<const ulonglong2*>(row + pl + 2 * h);
+                } else {
+                    ch.x = *reinterpret_cast<const f2p*>(row + 2 * h);
+                    cl.x = *reinterpret_cast<const f2p*>(row + pl + 2 * h);
+                }
+#pragma unroll
+                for (int t = 0; t < P; ++t) {
+                    df_mac2(sh[t][h], sl[t][h], xh[t], nxh[t], xl[t], ch.x, cl.x);
+                    if (h + 1 < H) df_mac2(sh[t][h + 1], sl[t][h + 1], xh[t], nxh[t], xl[t], ch.y, cl.y);
+                }
             }
         }
     }
     cp_async_wait_all();
 #pragma unroll
-    for (int h = 0; h < H; ++h) {
-        const float2 vh = upk2(sh[h]), vl = upk2(sl[h]);
-        if (2 * h < jn) out[(size_t)(j0 + 2 * h) * Ng + p] = df_to_double(vh.x, vl.x);
-        if (2 * h + 1 < jn) out[(size_t)(j0 + 2 * h + 1) * Ng + p] = df_to_double(vh.y, vl.y);
+    for (int t = 0; t < P; ++t) {
+        const int pt = p + t * NT;
+        if (pt >= Ng) break;
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            const float2 vh = upk2(sh[t][h]), vl = upk2(sl[t][h]);
+            if (2 * h < jn) out[(size_t)(j0 + 2 * h) * Ng + pt] = df_to_double(vh.x, vl.x);
+            if (2 * h + 1 < jn) out[(size_t)(j0 + 2 * h + 1) * Ng + pt] = df_to_double(vh.y, vl.y);
+        }
     }
 }
 
+template <int P>
 __global__ void __launch_bounds__(256) tsmm_df_kernel(TsmmArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* sC = reinterpret_cast<float*>(smem_raw);
@@ -601,20 +633,19 @@ __global__ void __launch_bounds__(256) tsmm_df_kernel(TsmmArgs a) {
         sC[pl + e] = v.y;
     }
     __syncthreads();
-    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= a.Ng) return;
+    const int Ng = (int)a.Ng, p = blockIdx.x * (256 * P) + threadIdx.x;
+    if (p >= Ng) return;
     const void* const* cols = a.colsIn + (size_t)b * a.ldcols;
     double* out = reinterpret_cast<double*>(a.out) + (size_t)b * a.ld_out_b;
     // per-thread input slots after the C planes (16-byte aligned)
     double* stg = reinterpret_cast<double*>(smem_raw + ((size_t)2 * pl * sizeof(float) + 15) / 16 * 16) + threadIdx.x;
-    const int nthr = blockDim.x;
     for (int j0 = 0; j0 < KOUT; j0 += 16) {
         const int jn = min(16, KOUT - j0);
-        switch ((jn + 3) / 4) {
-        case 1: tsmm_df_block<4>(cols, KIN, sC, pl, KP, j0, jn, p, a.Ng, out, stg, nthr); break;
-        case 2: tsmm_df_block<8>(cols, KIN, sC, pl, KP, j0, jn, p, a.Ng, out, stg, nthr); break;
-        case 3: tsmm_df_block<12>(cols, KIN, sC, pl, KP, j0, jn, p, a.Ng, out, stg, nthr); break;
-        default: tsmm_df_block<16>(cols, KIN, sC, pl, KP, j0, jn, p, a.Ng, out, stg, nthr); break;
+        switch ((jn + 1) / 2) {
+#define PR_TSMM_CASE(H_) case H_: tsmm_df_block<2 * H_, P>(cols, KIN, sC, pl, KP, j0, jn, p, Ng, out, stg); break;
+            PR_TSMM_CASE(1) PR_TSMM_CASE(2) PR_TSMM_CASE(3) PR_TSMM_CASE(4)
+            PR_TSMM_CASE(5) PR_TSMM_CASE(6) PR_TSMM_CASE(7) PR_TSMM_CASE(8)
+#undef PR_TSMM_CASE
         }
     }
 }
@@ -623,11 +654,21 @@ cudaError_t launch_tsmm(const TsmmArgs& a, bool in_f32, bool out_f32, cudaStream
     if (a.B <= 0 || a.maxKOUT <= 0) return cudaSuccess;
     dim3 grid((unsigned)((a.Ng + 255) / 256), a.B);
     const size_t cells = (size_t)a.maxKIN * ((a.maxKOUT + 3) / 4 * 4);
-    if (a.df && !in_f32 && !out_f32) {
-        const size_t smem = (2 * cells * sizeof(float) + 15) / 16 * 16 + (size_t)2 * TSMM_TG * 256 * sizeof(double);
-        if (smem > 48 * 1024)
-            cudaFuncSetAttribute((const void*)tsmm_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        tsmm_df_kernel<<<grid, 256, smem, st>>>(a);
+    if (a.df && !in_f32 && !out_f32 && a.Ng <= (1LL << 30)) {
+        // two points a thread where that leaves every SM four CTAs
+        int dev = 0, sms = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        const int P = (a.Ng + 511) / 512 * a.B >= 4LL * sms ? 2 : 1;
+        const size_t smem =
+            (2 * cells * sizeof(float) + 15) / 16 * 16 + (size_t)2 * TSMM_TG * P * 256 * sizeof(double);
+        const void* fn = P == 2 ? (const void*)tsmm_df_kernel<2> : (const void*)tsmm_df_kernel<1>;
+        if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (P == 2)
+            tsmm_df_kernel<2><<<dim3((unsigned)((a.Ng + 511) / 512), a.B), 256, smem, st>>>(a);
+        else
+            tsmm_df_kernel<1><<<grid, 256, smem, st>>>(a);
     } else if (in_f32 && out_f32) {
         tsmm_kernel<float, float, float><<<grid, 256, cells * sizeof(float), st>>>(a);
     } else if (!in_f32 && out_f32) {
