@@ -194,17 +194,30 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
+__device__ __forceinline__ void gdf_cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ const double* gdf_peer(const double* p, int rank) {
+    unsigned long long o;
+    asm volatile("mapa.u64 %0, %1, %2;" : "=l"(o) : "l"(reinterpret_cast<unsigned long long>(p)), "r"(rank));
+    return reinterpret_cast<const double*>(o);
+}
+
 template <int SUB>
-__global__ void __launch_bounds__(GDF_MAXTHR, 2) gram_df_kernel(GramArgs a, long long CH, int chunks) {
+__global__ void __launch_bounds__(GDF_MAXTHR, 2) gram_df_kernel(GramArgs a, long long CH, int chunks, int cl) {
     constexpr int GDF_SUB = SUB, GDF_LDP = SUB + 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nthr = blockDim.x, tid = threadIdx.x;
-    const int b = blockIdx.y, c = blockIdx.x;
+    // a cluster of cl CTAs shares a chunk's rows; its first CTA adds their sums
+    const int b = blockIdx.y, c = blockIdx.x / cl, rank = blockIdx.x - c * cl;
     const int KA = a.KA[b];
     const int KB = a.sym ? KA : a.KB[b];
     const int nout = a.sym ? KA * (KA + 1) / 2 : KA * KB;
-    const long long p_lo = (long long)c * CH;
-    const long long p_hi = min(a.Ng, p_lo + CH);
+    const int c_hi = (int)min(a.Ng, (long long)(c + 1) * CH);   // point indices fit 32 bits (launch_gram)
+    const int share = cl == 1 ? (int)CH : (((int)CH + cl - 1) / cl + SUB - 1) / SUB * SUB;
+    const int p_lo = min(c_hi, c * (int)CH + rank * share);
+    const int p_hi = min(c_hi, p_lo + share);
     const int ncA = gdf_cols(a.maxKA), ncB = a.sym ? 0 : gdf_cols(a.maxKB);
     const int plA = ncA * GDF_LDP, plB = ncB * GDF_LDP;
     double* rawA = reinterpret_cast<double*>(smem_raw);             // [ncA][GDF_SUB]
@@ -242,7 +255,7 @@ __global__ void __launch_bounds__(GDF_MAXTHR, 2) gram_df_kernel(GramArgs a, long
                     for (int r = 0; r < 2; ++r)
                         for (int s2 = 0; s2 < 2; ++s2) {
                             const int i = i0 + r, j = j0 + s2;
-                            if (i < KA && j < KA && i <= j)
+                            if (rank == 0 && i < KA && j < KA && i <= j)
                                 mypart[(size_t)i * a.maxKB + j] = (i == j && c == 0) ? 1.0 : 0.0;
                         }
                 }
@@ -283,10 +296,10 @@ __global__ void __launch_bounds__(GDF_MAXTHR, 2) gram_df_kernel(GramArgs a, long
         for (int r = 0; r < 2; ++r)
 #pragma unroll
             for (int q = 0; q < 2; ++q) sh[r][q] = sl[r][q] = Ah[r][q] = Al[r][q] = 0ull;
-        auto load = [&](double* raw, int ncols, int K, const void* const* cols, long long p0) {
+        auto load = [&](double* raw, int ncols, int K, const void* const* cols, int p0) {
             for (int e = tid; e < ncols * GDF_SUB; e += nthr) {
                 const int col = e / GDF_SUB, r = e - col * GDF_SUB;
-                const long long p = p0 + r;
+                const int p = p0 + r;
                 const bool ok = col < K && p < p_hi;
                 const double* src = ok ? reinterpret_cast<const double*>(cols[col]) + p : reinterpret_cast<const double*>(a.part);
                 cp_async8(raw + e, src, ok ? 8 : 0);
@@ -312,7 +325,7 @@ __global__ void __launch_bounds__(GDF_MAXTHR, 2) gram_df_kernel(GramArgs a, long
         if (!a.sym) load(rawB, kB, KB, colsB, p_lo);
         cp_async_commit();
         int nblk = 0;
-        for (long long p0 = p_lo; p0 < p_hi; p0 += GDF_SUB) {
+        for (int p0 = p_lo; p0 < p_hi; p0 += GDF_SUB) {
             cp_async_wait_all();
             __syncthreads();   // this block's rows landed; every thread is done with the planes
             convert(rawA, sA, plA, kA);
@@ -387,7 +400,28 @@ __global__ void __launch_bounds__(GDF_MAXTHR, 2) gram_df_kernel(GramArgs a, long
                 }
             }
         }
-        if (active && grp == 0) {
+        if (cl > 1) {
+            __syncthreads();   // the group sums are read
+            if (active && grp == 0 && rank > 0) {
+                double* d = sacc + (size_t)tid * 4;
+                d[0] = acc[0][0];
+                d[1] = acc[0][1];
+                d[2] = acc[1][0];
+                d[3] = acc[1][1];
+            }
+            gdf_cluster_sync();
+            if (active && grp == 0 && rank == 0) {
+                for (int k = 1; k < cl; ++k) {
+                    const double* d = gdf_peer(sacc + (size_t)tid * 4, k);
+                    acc[0][0] += d[0];
+                    acc[0][1] += d[1];
+                    acc[1][0] += d[2];
+                    acc[1][1] += d[3];
+                }
+            }
+            gdf_cluster_sync();   // the others' memory is free again
+        }
+        if (active && grp == 0 && rank == 0) {
 #pragma unroll
             for (int r = 0; r < 2; ++r)
 #pragma unroll
@@ -398,6 +432,7 @@ __global__ void __launch_bounds__(GDF_MAXTHR, 2) gram_df_kernel(GramArgs a, long
         }
         __syncthreads();   // the group sums are read: the buffers are free for the next pass
     }
+    if (rank > 0) return;
     gram_finish(a, b, chunks, KA, KB, nout);
 }
 
@@ -445,7 +480,7 @@ static cudaError_t gram_dispatch(const GramArgs& a, cudaStream_t st) {
 
 cudaError_t launch_gram(const GramArgs& a, bool a_f32, bool b_f32, cudaStream_t st) {
     if (a.B <= 0 || a.maxKA <= 0 || (!a.sym && a.maxKB <= 0)) return cudaSuccess;
-    if (a.df && !a_f32 && !b_f32) {
+    if (a.df && !a_f32 && !b_f32 && a.Ng <= (1LL << 30)) {
         const int thr = gram_df_threads(a);
         int sub = thr >= 256 ? 128 : 64;
         size_t smem = thr > 0 ? gram_df_smem(a, thr, sub) : 0;
@@ -459,10 +494,33 @@ cudaError_t launch_gram(const GramArgs& a, bool a_f32, bool b_f32, cudaStream_t 
             const void* fn = sub == 128 ? (const void*)gram_df_kernel<128> : (const void*)gram_df_kernel<64>;
             if (smem > 48 * 1024)
                 cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (sub == 128)
-                gram_df_kernel<128><<<dim3(chunks, a.B), thr, smem, st>>>(a, CH, chunks);
-            else
-                gram_df_kernel<64><<<dim3(chunks, a.B), thr, smem, st>>>(a, CH, chunks);
+            // Few items leave one CTA an SM or less, which waits for its loads and its barriers in
+            // turn: clusters of up to four CTAs share the chunks while all of them are resident
+            // (more chunks would lengthen the last CTA's sum over them).  The coarse update on 64^3
+            // with 16 columns, whose two Grams have one item each: 460 -> 429 us.
+            int cl = 1, dev = 0, sms = 0, occ = 0;
+            cudaError_t e = cudaGetDevice(&dev);
+            if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            if (e != cudaSuccess) return e;
+            const long long ctas = (long long)chunks * a.B;
+            if (ctas <= 2LL * sms && CH >= 4 * sub) {
+                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, thr, smem);
+                if (e != cudaSuccess) return e;
+                while (cl < 4 && (cl + 1) * ctas <= (long long)occ * sms) ++cl;
+            }
+            cudaLaunchConfig_t cfg{};
+            cudaLaunchAttribute at[1];
+            cfg.gridDim = dim3((unsigned)(chunks * cl), (unsigned)a.B);
+            cfg.blockDim = dim3((unsigned)thr);
+            cfg.dynamicSmemBytes = smem;
+            cfg.stream = st;
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = (unsigned)cl;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = cl > 1 ? 1 : 0;
+            e = cudaLaunchKernelEx(&cfg, sub == 128 ? gram_df_kernel<128> : gram_df_kernel<64>, a, CH, chunks, cl);
+            if (e != cudaSuccess) return e;
             ++g_launch_count;
             return cudaGetLastError();
         }
