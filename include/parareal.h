@@ -152,9 +152,10 @@ enum pr_method { PR_METHOD_ADAPTIVE = 0, PR_METHOD_PARAREAL_I = 1, PR_METHOD_PAR
  * FP32 pipe (up to 126 columns, windows wider than 54 columns in several passes over the
  * data; FP64 beyond).  PR_GRAM_TENSOR: the tensor cores, with the values cut into
  * error-free BF16 digits (FP64-accurate, see pr_op_gram; up to 64 columns, double-float
- * beyond).  PR_GRAM_AUTO: the tensor cores for snapshot windows of 20..32 columns (where
- * the narrow tensor-core form is faster) and 55..64 columns (where the double-float
- * kernel would need two passes), double-float otherwise (and for the Cholesky-QR Grams,
+ * beyond).  PR_GRAM_AUTO: the tensor cores for snapshot windows of 20..32 and 55..64
+ * columns, and of 33..54 where a call has 262144 points or more (and the context's
+ * spin_limit is 4096 or more: double-float waits for nothing), where they are faster;
+ * double-float otherwise (and for the Cholesky-QR Grams,
  * whose column counts are POD dimensions known only on the device).  The FP64 mode always
  * forms its Grams in FP64. */
 enum pr_gram_mode { PR_GRAM_AUTO = 0, PR_GRAM_DF = 1, PR_GRAM_TENSOR = 2 };

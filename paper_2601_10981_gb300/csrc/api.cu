@@ -400,8 +400,8 @@ pr_status cols_contig(pr_ctx* c, const char* base, size_t bstride_bytes, const i
 // ortho_blocks: the snapshot columns are blocks of orthonormal bases (c->colblk says
 // which); the FP32 mode then takes their diagonal Gram blocks as the identity.
 // Symmetric Grams of the FP32 mode: on the tensor cores (error-free BF16 digit products,
-// FP64-accurate; gram_tc.cu) for 55..64 columns, which the double-float kernel does not
-// take (gram_mode PR_GRAM_AUTO), for every width up to 64 (PR_GRAM_TENSOR), or never
+// FP64-accurate; gram_tc.cu) for windows of 20..64 columns (gram_mode PR_GRAM_AUTO), for every
+// width up to 64 (PR_GRAM_TENSOR), or never
 // (PR_GRAM_DF); every other Gram runs in double-float or FP64.
 // k_exact: every item has maxKA columns (a snapshot window), not a cap on a POD dimension
 // that lives on the device; the automatic choice of the tensor cores needs the column
@@ -413,9 +413,13 @@ cudaError_t gram_auto(pr_ctx* c, const GramArgs& ga, bool in_f32, bool k_exact) 
     // measured crossovers against the double-float kernel (64 items x 262,144 points, wall
     // time incl. the column-maximum pass): the narrow tensor form (<= 32 columns) wins from
     // 20 columns (20: 2.7 vs 3.0 ms, 32: 3.3 vs 6.9 ms; 16: 2.1 vs 1.9), the wide one
-    // (33..64) beyond the double-float kernel's 384 output tiles a pass (55 columns)
+    // (33..64) from 262,144 points in all (op_gram, 33 and 54 columns: 64^3 x 16 1.07 vs 1.81
+    // and 1.22 vs 4.07 ms, 32^3 x 16 0.23 vs 0.30 and 0.27 vs 0.66, 64^3 x 1 0.19 vs 0.21 and
+    // 0.28 vs 0.39; 32^3 x 1 0.13 vs 0.09 and 0.19 vs 0.14), and beyond the double-float
+    // kernel's 384 output tiles a pass (55 columns) always.  Double-float waits for nothing: a
+    // context whose waits may not last (spin_limit below a few milliseconds) keeps it there.
     const bool narrow = ga.maxKA >= 20 && ga.maxKA <= 32;
-    const bool wide = ga.maxKA > 54;
+    const bool wide = ga.maxKA > 54 || (ga.maxKA > 32 && ga.B * ga.Ng >= 262144 && c->o.spin_limit >= 4096);
     if (fits && (mode == PR_GRAM_TENSOR || (mode == PR_GRAM_AUTO && k_exact && (narrow || wide))))
         return launch_gram_tc(ga, c->colmax, gram_tc_max_cols(), c->derr, c->o.spin_limit, c->st);
     return launch_gram(ga, in_f32, in_f32, c->st);

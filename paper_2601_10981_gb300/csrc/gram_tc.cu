@@ -37,7 +37,8 @@
 // is six MMAs.  Every wait on an mbarrier is bounded: on time-out the kernel records
 // PR_ERR_TIMEOUT, waits (bounded) for its MMAs in flight, frees its tensor memory and
 // returns.  Column maxima come from a pre-pass (colmax_kernel).
-// TCFIG
+// Four windows of 64 columns on 128^3: 6.5 -> 2.4 ms (one: 1.72 -> 0.60 ms, the tensor pipe 71 %
+// busy, it was 22; a POD call 18.2 -> 12.9 ms).
 #include "pr_internal.cuh"
 
 #include <cuda_bf16.h>
@@ -978,10 +979,16 @@ cudaError_t launch_gram_tc(const GramArgs& a, unsigned long long* colmax, int ld
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // Units of about 16384 points, as many as fill whole waves of the grid, but one wave at least
+    // (short units pay a read-back, the partials' fences and the last CTA's sum over them: 16
+    // windows of 33 columns on 32^3, 791 us in units of 320 points, 230 us in one wave; 16 of 54
+    // on 64^3, 2.64 and 1.22 ms)
+    const long long waves = std::max<long long>(1, a.B * a.Ng / 16384 / std::max(1, sms));
+    const int cw = (int)std::min<long long>(chunks, std::max<long long>(1, waves * sms / a.B));
     if (a.maxKA <= N2_COLS && chunks >= 2) {
-        // narrow form: units of U points (at least two per partial slot of the other Gram
-        // kernels, since a unit's partial is K x K 128-bit integers)
-        const int ctc = chunks / 2;
+        // narrow form: at most one unit for two partial slots of the other Gram kernels, since a
+        // unit's partial is K x K 128-bit integers
+        const int ctc = std::min(cw, chunks / 2);
         const long long U2 = ((a.Ng + ctc - 1) / ctc + N2_PTS - 1) / N2_PTS * N2_PTS;
         const int chunks2 = (int)((a.Ng + U2 - 1) / U2);
         e = cudaFuncSetAttribute((const void*)gram_tc32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -992,11 +999,7 @@ cudaError_t launch_gram_tc(const GramArgs& a, unsigned long long* colmax, int ld
         ++g_launch_count;
         return cudaGetLastError();
     }
-    // wide form, one CTA an SM (the tiles take all 512 tensor-memory columns, the ring most of the
-    // shared memory): chunks that fill whole waves of the grid where there are several waves
-    // (4 windows of 128^3: 512 units of 16384 points were 3.4 waves of 152)
-    const int waves = std::max(1, a.B * chunks / std::max(1, sms));
-    const int cw = std::min(chunks, std::max(1, (int)((long long)waves * sms / a.B)));
+    // wide form, one CTA an SM (the tiles take all 512 tensor-memory columns)
     const int CHw = (int)(((a.Ng + cw - 1) / cw + TC_PTS - 1) / TC_PTS * TC_PTS);
     const int chunksw = (int)((a.Ng + CHw - 1) / CHw);
     e = cudaFuncSetAttribute((const void*)gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);

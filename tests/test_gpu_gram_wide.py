@@ -38,3 +38,26 @@ def test_wide_tensor_gram(gpu, n, K, B):
             cut = 2.0 ** -53 * (np.abs(x).sum() * np.abs(y).max() + np.abs(y).sum() * np.abs(x).max())
             tol = cut + 8 * 2.0 ** -57 * Ng * mx + 128 * 2.0 ** -53 * np.abs(x * y).sum()
             assert abs(G[b, i, j] - ref) <= tol, (b, i, j, G[b, i, j], ref, tol)
+
+
+# 33 to 54 columns: the tensor cores from 262,144 points in all, double-float below and where
+# waits may not last
+@pytest.mark.parametrize("n,B,K,opts", [(64, 1, 33, {}), (63, 1, 40, {}), (63, 2, 40, {}), (64, 1, 54, {"spin_limit": 0}),
+                                        (64, 1, 54, {"spin_limit": 4096})])
+def test_pod_of_middle_widths(gpu, n, B, K, opts):
+    bd, torch = gpu
+    w = pi.Workload("mid", n, pi.Flow("abc"), 0.05, 1.0, B, 1.0 / (B * (K - 1)), n_snap=K, m_cap=16)
+    s = bd.Parareal.from_workload(w, precision=bd.PR_FP32, **opts)
+    sig = np.logspace(0.0, -1.0, K)
+    gap = float(np.min(-np.diff(sig ** 2)))
+    tol = 16.0 * K * 3.6e-15 / gap + 1e-12   # double-float accuracy over the eigenvalues' gap
+    rng = np.random.default_rng(n + K)
+    Q = [np.linalg.qr(rng.standard_normal((n ** 3, K)))[0] for _ in range(B)]
+    Y = np.linalg.qr(rng.standard_normal((K, K)))[0]
+    W = np.ascontiguousarray(np.stack([((q * sig) @ Y.T).T for q in Q]))
+    R, m = s.op_pod(torch.from_numpy(W).cuda().reshape(B, K, n, n, n), 1.0, 16)
+    R = R.cpu().numpy().reshape(B, -1, n ** 3)
+    s.close()
+    for b in range(B):
+        assert m[b] == 16
+        assert np.abs(np.abs(R[b] @ Q[b][:, :16]) - np.eye(16)).max() < tol, b
