@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
     // for the plane at hand and the next, in y ([plane & 1][+-][x]).  GB300's FP64 pipe (2 FMAs
     // a cycle and SM) bounds the FP64 mode, and forming the weights at each point took half of
     // A's operations: A is now 7 FMAs a point, and <rhat, t> joins the products
-    // of the t phase, so the update phase needs none.  64^3, 16 subintervals x 32 steps: 68.0 ->
+    // of the t phase, so the update phase needs none.  64^3, 64 subintervals x 16 steps: 68.0 ->
     // 61.1 ms (the pipe 81 % busy); 96^3 x 8 x 10: 22.7 -> 18.0 ms; 128^3 x 8 x 10: 42.6 -> 38.1.
     double* wz = ringd + (DF ? 0 : FINE_SLOTS * (a.TY + 2) * n);
     double* wy = wz + 2 * a.TY * n;
