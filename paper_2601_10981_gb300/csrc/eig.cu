@@ -20,8 +20,8 @@
 //     operations deep in place of four divisions and roots.
 // POD of 64 windows of 32 snapshots on 64^3 (C = 2): 11.1 -> 9.7 ms, the solver 3.3 ms of it before;
 // of four windows of 64 on 128^3 (C = 8): 27.2 -> 18.2 ms, the solver 12.1 ms of it before.
-// A round takes 5,100 cycles (K = 32, C = 2 or K = 64, C = 8; 12,000 to 20,000 before): 2,500 to
-// 3,400 for the blocks, 400 to 900 to arrive at the barrier, 1,900 for the angles.
+// A round takes 5,100 cycles (K = 32, C = 2 or K = 64, C = 8; about 12,000 at K = 64 before): 2,500
+// to 3,400 for the blocks, 400 to 900 to arrive at the barrier, 1,900 for the angles.
 #include "df.cuh"
 #include "pr_internal.cuh"
 
