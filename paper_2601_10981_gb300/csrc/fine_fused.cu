@@ -233,6 +233,16 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         sh.fail = 0;
     }
+    // What the launch after this one has to do for an item: nothing, until the item is done here.
+    // Written before anything can wait: a wait that gives up then leaves no entry of an earlier
+    // launch, or of uninitialised memory, behind.
+    if (q == 0 && threadIdx.x == 0) {
+        for (int b = g; b < a.B; b += a.numGroups) {
+            int jb = 0, lb = b;
+            while (jb + 1 < a.njobs && lb >= a.jobs[jb].B) lb -= a.jobs[jb++].B;
+            a.jobs[jb].resume[lb] = 0;
+        }
+    }
     __syncthreads();
     auto wait_full = [&](int i, unsigned parity) {
         if (!mbar_wait(&sh.full[i], parity, a.spin_limit)) {

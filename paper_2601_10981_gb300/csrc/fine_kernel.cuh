@@ -770,8 +770,8 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
         const FineJob& J = a.jobs[jb];
         // an item that fused_kernel left (J.resume): from its step j0 on, its state in u_out
         const int j0 = J.resume ? J.resume[lb] : 1;
-        if (j0 == 0) continue;
         const int S = J.S, dM = J.dM, n_snap = J.n_snap;
+        if (J.resume && (j0 < 1 || j0 > S)) continue;   // 0: nothing is left
         const double* u_in = (J.resume ? J.u_out : J.u_in) + (size_t)lb * Ng;
         double* snap_b = J.snap ? reinterpret_cast<double*>(J.snap) + (size_t)lb * n_snap * Ng : nullptr;
         long long its_total = 0;

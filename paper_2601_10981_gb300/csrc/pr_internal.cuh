@@ -188,8 +188,9 @@ struct FineJob {
     int* its_total;     // [B]
     int* its_max;       // [B]
     int B;
-    int* resume;        // [B] the step at which fused_kernel left an item, 0: none; null: a launch
-                        // of fine_kernel that does all steps of all items
+    int* resume;        // [B] the step at which fused_kernel left an item, 0: none (fused_kernel
+                        // writes every entry before it can wait); null: a launch of fine_kernel
+                        // that does all steps of all items
     const void* pert;   // stored velocity perturbation [3][Ng] in the Krylov type (float in
                         // the FP32 mode, double in FP64), unscaled, or nullptr
 };
