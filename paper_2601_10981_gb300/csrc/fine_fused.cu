@@ -48,12 +48,14 @@ constexpr int FUSED_RSLOTS = 6;   // planes of r in the krylov pass, three of th
 // relative size below which a norm formed from products is not trusted (the products, summed in
 // floats, hold ~1e-6)
 constexpr double FUSED_CANCEL = 1e-4;
+constexpr long long FUSED_DRAIN = 1 << 20;   // tries of a wait for copies in flight before leaving
 constexpr int FUSED_AGAIN = 2;   // further iterations of an item's steps before it is left to fine_kernel
 
 struct FusedShared : FineShared {
     float wred[5 * 32];
     float al, om, ga;   // alpha, omega, 1 - alpha of the last iteration: delta + al r + om (ga r - al q)
-    int ok, fail, its_max;
+    int ok, its_max;
+    int gave_up[2];     // a wait of an even, an odd plane gave up
     long long its_total;
     unsigned long long full[FUSED_SSLOTS + FUSED_RSLOTS];   // mbarriers: copies landed
 };
@@ -137,7 +139,7 @@ __device__ __forceinline__ bool group_reduce(float (&v)[NQ], FusedShared& sh, do
         asm volatile("fence.proxy.async.global;" ::: "memory");
     }
     __syncthreads();
-    return sh.ok != 0 && sh.fail == 0;
+    return sh.ok != 0;
 }
 
 // One contiguous asynchronous copy, global to shared, counted on an mbarrier, and its
@@ -231,7 +233,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
         for (int i = 0; i < FUSED_SSLOTS + FUSED_RSLOTS; ++i)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(&sh.full[i])));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        sh.fail = 0;
+        sh.gave_up[0] = sh.gave_up[1] = 0;
     }
     // What the launch after this one has to do for an item: nothing, until the item is done here.
     // Written before anything can wait: a wait that gives up then leaves no entry of an earlier
@@ -244,10 +246,24 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
         }
     }
     __syncthreads();
-    auto wait_full = [&](int i, unsigned parity) {
+    // Waits for a slot's copies.  One that gives up says so in the entry of its plane's parity, which
+    // is read after the plane's barrier and written again two barriers later, so that all threads
+    // decide alike: they fill no slot again, wait for the copies in flight (`drain`: `count` slots of a
+    // ring of `nring` from slot sl on, sl's landing of parity ph) and leave.  The group's other CTAs give
+    // up at their next barrier.  (A vote at that barrier instead, __syncthreads_or, cost 4 %: 64^3 x 64 x 157 steps 27.9 -> 29.0 ms.)
+    auto wait_full = [&](int i, unsigned parity, int plane) {
         if (!mbar_wait(&sh.full[i], parity, a.spin_limit)) {
             record_error(a.err, DERR_TIMEOUT);
-            sh.fail = 1;
+            sh.gave_up[plane & 1] = 1;
+        }
+    };
+    auto drain = [&](int first, int nring, int sl, unsigned ph, int count) {
+        for (; count > 0; --count) {
+            mbar_wait(&sh.full[first + sl], ph, FUSED_DRAIN);
+            if (++sl == nring) {
+                sl = 0;
+                ph ^= 1;
+            }
         }
     };
     auto wrapz = [&](int z) { return z < 0 ? z + n : (z >= n ? z - n : z); };
@@ -432,7 +448,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
                     for (int u = 0; u < FU; ++u) oc[u] = op[u] = dc[u] = fc[u] = zero4();
                     float *rp = ring, *rq = ring + 2 * PL;   // ring planes of zp and of the stencil
                     for (int zp = zlo - 1; zp <= zhi; ++zp) {
-                        wait_full(ss, sph);
+                        wait_full(ss, sph, zp);
                         const float* sl = slots + ss * (fs.slot / 4);
                         const bool inside = zp >= zlo && zp < zhi;
                         P4 dn[FU], fn[FU];
@@ -477,7 +493,8 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
                             st4(rp + o, operand(sl, o, h_, l_, d_));
                         }
                         __syncthreads();
-                        if (zp + NS <= zhi) issue(zp + NS, ss);
+                        const int gave_up = sh.gave_up[zp & 1];
+                        if (zp + NS <= zhi && !gave_up) issue(zp + NS, ss);
                         if (++ss == NS) {
                             ss = 0;
                             sph ^= 1;
@@ -522,6 +539,11 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
                         }
                         rq = rp;
                         rp = rp == ring + 2 * PL ? ring : rp + PL;
+                        if (gave_up) {   // planes zp .. zp + NS - 1 were on their way; ss is zp's next slot
+                            const int sl = ss == 0 ? NS - 1 : ss - 1;
+                            drain(0, NS, sl, ss == 0 ? sph ^ 1u : sph, min(NS, zhi - zp + 1));
+                            return;
+                        }
                     }
                     __syncthreads();   // the next tile rewrites the ring's first planes
                 }
@@ -628,16 +650,16 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
                             sl = next(sl);
                         }
                     }
-                    auto landed = [&]() {   // waits for the next plane; its slot
+                    auto landed = [&](int z) {   // waits for the next plane, in plane z's turn; its slot
                         const int sl = rs;
-                        wait_full(FUSED_SSLOTS + sl, rph);
+                        wait_full(FUSED_SSLOTS + sl, rph, z);
                         if (++rs == FUSED_RSLOTS) {
                             rs = 0;
                             rph ^= 1;
                         }
                         return sl;
                     };
-                    int sm = 0, sc = landed(), sp = landed();
+                    int sm = 0, sc = landed(zlo - 1), sp = landed(zlo - 1);
                     P4 rm[FU], rv[FU], rp[FU], qm[FU], qc[FU], qp[FU];   // r at z-1, z, z+1; q at z-2, z-1, z
 #pragma unroll
                     for (int u = 0; u < FU; ++u) {
@@ -650,7 +672,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
                     for (int z = zlo - 1; z <= zhi; ++z) {
                         sm = sc;
                         sc = sp;
-                        sp = landed();
+                        sp = landed(z);
                         const int zw = wrapz(z);
                         const float ax = tabk[TXZ * n + zw], ay0 = tabk[TYZ * n + zw];
                         const float* cpl = slots + sc * RP_;
@@ -691,7 +713,8 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
                                                   tabk[TXY * n + yy] + tabk[TXZ * n + zw], ay0, pack4(vy), pack4(vp), pack4(vm)));
                         }
                         __syncthreads();
-                        if (warp == 0 && z - 1 + FUSED_RSLOTS <= zhi + 1) issue(z - 1 + FUSED_RSLOTS, sm);
+                        const int gave_up = sh.gave_up[z & 1];
+                        if (warp == 0 && z - 1 + FUSED_RSLOTS <= zhi + 1 && !gave_up) issue(z - 1 + FUSED_RSLOTS, sm);
                         if (z > zlo) {   // q2 at z - 1
 #pragma unroll
                             for (int u = 0; u < FU; ++u) {
@@ -711,6 +734,10 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
                         aym = ay0;
                         qcl = qpl;
                         qpl = qpl == ring + 2 * PL ? ring : qpl + PL;
+                        if (gave_up) {   // planes z - 1 .. z + 4 were on their way, from slot sm on
+                            drain(FUSED_SSLOTS, FUSED_RSLOTS, sm, sm < rs ? rph : rph ^ 1u, min(FUSED_RSLOTS, zhi + 3 - z));
+                            return;
+                        }
                     }
                     __syncthreads();
                 }

@@ -14,6 +14,15 @@ pytestmark = pytest.mark.gpu
 PR_ERR_TIMEOUT = 6
 
 
+def filled(bd, torch, w, fill, **kw):
+    """A context whose workspace holds `fill` in every byte when it is bound."""
+    s = bd.Parareal.from_workload(w, precision=bd.PR_FP32, workspace=False, **kw)
+    n = s.workspace_bytes()
+    s.ws = torch.full((n + 256,), fill, dtype=torch.uint8, device="cuda")
+    s._check(s._lib.pr_bind_workspace(s.ctx, ctypes.c_void_p((s.ws.data_ptr() + 255) // 256 * 256), n))
+    return s
+
+
 def fine_into(s, torch, u, steps, dM, n_snap):
     """op_fine into buffers with guard words around the snapshots; its status and results."""
     B, Ng = u.shape[0], u[0].numel()
@@ -42,8 +51,7 @@ def test_two_pass_waits_that_run_out(gpu, limit, G, dt):
     assert st == 0
     s.close()
     for fill in (0x80, 0x01):   # negative and large positive entries
-        s = bd.Parareal.from_workload(w, precision=bd.PR_FP32, group_ctas=G, spin_limit=limit)
-        s.ws.fill_(fill)
+        s = filled(bd, torch, w, fill, group_ctas=G, spin_limit=limit)
         s.set_initial(u[0].cpu().numpy(), w.f())
         for _ in range(2):      # the second call finds what the first one left
             st, out, snap = fine_into(s, torch, u, steps, dM, n_snap)
@@ -53,9 +61,32 @@ def test_two_pass_waits_that_run_out(gpu, limit, G, dt):
                     assert rel(out[b], ref[b]) < steps * step_tol(w, dt), b
                     assert rel(snap[b], sref[b]) < steps * step_tol(w, dt), b
         s.close()
-    s = bd.Parareal.from_workload(w, precision=bd.PR_FP32, group_ctas=G)
-    s.ws.fill_(0x80)
+    s = filled(bd, torch, w, 0x80, group_ctas=G)
     s.set_initial(u[0].cpu().numpy(), w.f())
     st, out, snap = fine_into(s, torch, u, steps, dM, n_snap)
     assert st == 0 and np.array_equal(out, ref) and np.array_equal(snap, sref)
     s.close()
+
+
+# one CTA a group waits for its copies only: at one poll a copy that has not landed ends the
+# launch, with others of it in flight (one tile of 40 rows, tiles of 16)
+@pytest.mark.parametrize("n,steps", [(40, 6), (128, 4)])
+def test_two_pass_copies_in_flight_when_a_wait_gives_up(gpu, n, steps):
+    bd, torch = gpu
+    B, dt = 6, 5e-4
+    w = pi.Workload("two", n, pi.Flow("abc"), 0.005, B * 10 * dt, B, dt, n_snap=0, m_cap=4)
+    u = torch.from_numpy(np.stack([pi.initial_state(n, seed=30 + b) for b in range(B)])).cuda()
+    s = filled(bd, torch, w, 0x80, group_ctas=1)
+    s.set_initial(u[0].cpu().numpy(), None)
+    st, ref, _ = fine_into(s, torch, u, steps, 1, 2)
+    assert st == 0
+    t = filled(bd, torch, w, 0x80, group_ctas=1, spin_limit=1)
+    t.set_initial(u[0].cpu().numpy(), None)
+    for _ in range(3):
+        st, out, _ = fine_into(t, torch, u, steps, 1, 2)
+        assert st == PR_ERR_TIMEOUT or (st == 0 and rel(out, ref) < steps * step_tol(w, dt)), st
+        assert fine_into(s, torch, u, steps, 1, 2)[0] == 0   # the device is as it was
+    st, again, _ = fine_into(s, torch, u, steps, 1, 2)
+    assert st == 0 and np.array_equal(again, ref)
+    s.close()
+    t.close()
