@@ -266,16 +266,16 @@ __global__ void __launch_bounds__(512, 1) fine_chip_kernel(FineArgs a, ChipPlan 
     };
 
     chip_cluster_sync();   // every CTA of the cluster runs: its shared memory may be written
-    // The products of the second half of an iteration.  <rhat, s> = rho - alpha <rhat, v> is
-    // zero up to rounding by the choice of alpha; the FP32 mode, whose alpha is rounded to
-    // float, takes it into account, the FP64 mode does without.
-    constexpr int NQ2 = DF ? 5 : 4;
-    auto dots2 = [](KT (&s)[NQ2], KT tv, KT sv, KT hv) {
+    // The products of the second half of an iteration.  <rhat, s> = rho - alpha <rhat, v> is zero
+    // by the choice of alpha, but only as far as rho is <rhat, r>: taken as zero, rho keeps the rounding
+    // of the first iteration while <rhat, r> falls with the residual, and the FP64 mode no longer
+    // converged from about nine iterations a step on.
+    auto dots2 = [](KT (&s)[5], KT tv, KT sv, KT hv) {
         s[0] += tv * sv;
         s[1] += tv * tv;
         s[2] += sv * sv;
         s[3] += hv * tv;
-        if constexpr (NQ2 == 5) s[4] += hv * sv;
+        s[4] += hv * sv;
     };
     for (int b = cl; b < a.B; b += gridDim.x / C) {
         int jb = 0, lb = b;
@@ -512,13 +512,13 @@ __global__ void __launch_bounds__(512, 1) fine_chip_kernel(FineArgs a, ChipPlan 
                         }
                     }
                     __syncthreads();
-                    KT acc[NQ2] = {};
+                    KT acc[5] = {};
                     stencil(R, [&](int o, int z, int y, int x0, const Nb7<KT, W>& q) {
                         const Vec<KT, W> tv = applyA(o, z, y, x0, q);
                         vstore(T + own + o, tv);
                         push(Tb, Ta, o, tv);
                         const Vec<KT, W> hv = vload<KT, W>(first ? P + own + o : RH + o);
-                        KT s[NQ2] = {};
+                        KT s[5] = {};
 #pragma unroll
                         for (int e = 0; e < W; ++e) {
                             if constexpr (W == 1) {
@@ -529,7 +529,7 @@ __global__ void __launch_bounds__(512, 1) fine_chip_kernel(FineArgs a, ChipPlan 
                         }
                         if constexpr (W > 1) {
 #pragma unroll
-                            for (int k = 0; k < NQ2; ++k) acc[k] += s[k];
+                            for (int k = 0; k < 5; ++k) acc[k] += s[k];
                         }
                     });
                     reduce(acc, [&]() {
@@ -551,7 +551,7 @@ __global__ void __launch_bounds__(512, 1) fine_chip_kernel(FineArgs a, ChipPlan 
                                     act2 = CHIP_HALF;
                                 } else {
                                     const double rr1 = fma(-om, ts, ss);                    // ||s - omega t||^2
-                                    const double rho_new = DF ? fma(-om, sh.tot[3], sh.tot[4]) : -om * sh.tot[3];   // <rhat, r>
+                                    const double rho_new = fma(-om, sh.tot[3], sh.tot[4]);   // <rhat, r>
                                     if (!chip_finite(rr1)) {
                                         sh.status = DERR_NONFINITE;
                                         act2 = CHIP_FULL;

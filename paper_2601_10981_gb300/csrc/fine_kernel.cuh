@@ -32,6 +32,7 @@
 //   ph1   : p = r + beta (p' - omega v'),  v = A p;                  <rhat, v>
 //   ph2   : s = r - alpha v,               t = A s;        <t,s>, <t,t>, <s,s>
 //   ph3   : delta += alpha p + omega s,    r = s - omega t;      <rhat,r>, <r,r>
+// (FP64 implicit modes: <rhat,t>, <rhat,s> in ph2 in place of ph3's products)
 // p and s are recomputed at the 6 neighbours instead of being stored, p/v alternate
 // between two buffers so that neighbours read the previous iterate.
 // The persistent fine-sweep kernel (implicit Euler with BiCGStab per step, or explicit
@@ -391,7 +392,7 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
     // FP64 implicit modes: weights of A = I + dt L at the neighbours in z ([+-][tile row][x]) and,
     // for the plane at hand and the next, in y ([plane & 1][+-][x]).  GB300's FP64 pipe (2 FMAs
     // a cycle and SM) bounds the FP64 mode, and forming the weights at each point took half of
-    // A's operations: A is now 7 FMAs a point, and <rhat, t> joins the products
+    // A's operations: A is now 7 FMAs a point, and <rhat, t> and <rhat, s> join the products
     // of the t phase, so the update phase needs none.  64^3, 64 subintervals x 16 steps: 68.0 ->
     // 61.1 ms (the pipe 81 % busy); 96^3 x 8 x 10: 22.7 -> 18.0 ms; 128^3 x 8 x 10: 42.6 -> 38.1.
     double* wz = ringd + (DF ? 0 : FINE_SLOTS * (a.TY + 2) * n);
@@ -422,7 +423,7 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
     KT* t = Wk + 7 * Ng;
     double* ust = a.ust + (size_t)g * 2 * Ng;
     unsigned* bar = a.bar + 2 * g;
-    double* part = a.part;  // [2][4][grid]
+    double* part = a.part;  // [2][5][grid]
     const int g0 = g * G;
     int ph = 0;
 
@@ -754,10 +755,10 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
         acc.flush();
         cta_sum<KT, NQ>(acc, sh.red);
         if (threadIdx.x == 0) {
-            for (int qq = 0; qq < NQ; ++qq) part[(size_t)((ph & 1) * 4 + qq) * grid + blockIdx.x] = acc.d[qq];
+            for (int qq = 0; qq < NQ; ++qq) part[(size_t)((ph & 1) * 5 + qq) * grid + blockIdx.x] = acc.d[qq];
         }
         if (!group_barrier(bar, G, a.spin_limit, a.err)) return false;
-        group_sums(part + (size_t)(ph & 1) * 4 * grid, grid, g0, G, NQ, sh.sums, post);
+        group_sums(part + (size_t)(ph & 1) * 5 * grid, grid, g0, G, NQ, sh.sums, post);
         ++ph;
         return true;
     };
@@ -1228,10 +1229,13 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
                 // ---------------- ph2: s = r - alpha v, t = A s
                 {
                     const KT al = (KT)sh.alpha;
-                    // FP64: <rhat, t> too, from which beta and the stopping test follow without
-                    // the products of the update pass: <rhat, s> = rho - alpha <rhat, v> is zero
-                    // up to rounding, so <rhat, r> = -omega <rhat, t>, and ||r||^2 = <s,s> - omega <t,s>
-                    constexpr int NQ2 = DF ? 3 : 4;
+                    // FP64: <rhat, t> and <rhat, s> too, from which beta and the stopping test follow
+                    // without the products of the update pass: <rhat, r> = <rhat, s> - omega <rhat, t>,
+                    // ||r||^2 = <s,s> - omega <t,s>.  (<rhat, s> is zero by the choice of alpha, but
+                    // only as far as rho is <rhat, r>: taken as zero, rho keeps the rounding of the first
+                    // iteration while <rhat, r> falls with the residual, and steps of about nine
+                    // iterations or more no longer converged.)
+                    constexpr int NQ2 = DF ? 3 : 5;
                     Acc<KT, NQ2> acc;
                     acc.init();
                     march(true, ringk,
@@ -1256,7 +1260,10 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
                                   acc.f[0] += tv.v[e] * q7.c.v[e];
                                   acc.f[1] += tv.v[e] * tv.v[e];
                                   acc.f[2] += q7.c.v[e] * q7.c.v[e];
-                                  if constexpr (!DF) acc.f[3] += hv.v[e] * tv.v[e];
+                                  if constexpr (!DF) {
+                                      acc.f[3] += hv.v[e] * tv.v[e];
+                                      acc.f[4] += hv.v[e] * q7.c.v[e];
+                                  }
                               }
                               acc.tick();
                           });
@@ -1275,7 +1282,7 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
                     sh.flag = half;
                     if constexpr (!DF) {   // 0: go on, 1: delta += alpha p only, 2: the step is done
                         if (!half && sh.status == 0) {
-                            const double rr1 = fma(-sh.omega, ts, ss), rho_new = -sh.omega * s[3];
+                            const double rr1 = fma(-sh.omega, ts, ss), rho_new = fma(-sh.omega, s[3], s[4]);
                             sh.flag = 2;
                             if (!isfinite(rr1)) sh.status = DERR_NONFINITE;
                             else if (sqrt(fmax(rr1, 0.0)) <= sh.thr) {}
