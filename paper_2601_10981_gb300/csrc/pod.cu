@@ -204,29 +204,20 @@ __device__ __forceinline__ const double* gdf_peer(const double* p, int rank) {
     return reinterpret_cast<const double*>(o);
 }
 
-constexpr int GDF_SHARES = 3;
-// Rows of a share of a chunk of CH rows: whole blocks of sub.
-__host__ __device__ inline int gdf_share(int CH, int sub) {
-    return CH < 4 * sub ? CH : ((CH + GDF_SHARES - 1) / GDF_SHARES + sub - 1) / sub * sub;
-}
-
 template <int SUB>
-__global__ void __launch_bounds__(GDF_MAXTHR, 2) gram_df_kernel(GramArgs a, long long CH, int chunks, int cl,
-                                                               int park) {
+__global__ void __launch_bounds__(GDF_MAXTHR, 2) gram_df_kernel(GramArgs a, long long CH, int chunks, int cl) {
     constexpr int GDF_SUB = SUB, GDF_LDP = SUB + 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nthr = blockDim.x, tid = threadIdx.x;
-    // A chunk's rows are summed in GDF_SHARES shares (one if it is short), which are added in order,
-    // by one CTA or by a cluster with a share each (cl = GDF_SHARES), whose first CTA adds them: the
-    // sums are the same, so an item's Gram does not depend on how many items share the launch.
+    // a cluster of cl CTAs shares a chunk's rows; its first CTA adds their sums
     const int b = blockIdx.y, c = blockIdx.x / cl, rank = blockIdx.x - c * cl;
     const int KA = a.KA[b];
     const int KB = a.sym ? KA : a.KB[b];
     const int nout = a.sym ? KA * (KA + 1) / 2 : KA * KB;
     const int c_hi = (int)min(a.Ng, (long long)(c + 1) * CH);   // point indices fit 32 bits (launch_gram)
-    const int share = gdf_share((int)CH, SUB);
+    const int share = cl == 1 ? (int)CH : (((int)CH + cl - 1) / cl + SUB - 1) / SUB * SUB;
     const int p_lo = min(c_hi, c * (int)CH + rank * share);
-    const int p_hi = cl == 1 ? c_hi : min(c_hi, p_lo + share);
+    const int p_hi = min(c_hi, p_lo + share);
     const int ncA = gdf_cols(a.maxKA), ncB = a.sym ? 0 : gdf_cols(a.maxKB);
     const int plA = ncA * GDF_LDP, plB = ncB * GDF_LDP;
     double* rawA = reinterpret_cast<double*>(smem_raw);             // [ncA][GDF_SUB]
@@ -333,14 +324,7 @@ __global__ void __launch_bounds__(GDF_MAXTHR, 2) gram_df_kernel(GramArgs a, long
         load(rawA, kA, KA, colsA, p_lo);
         if (!a.sym) load(rawB, kB, KB, colsB, p_lo);
         cp_async_commit();
-        // a thread's sum over a share; the earlier shares' wait in shared memory (registers are short)
-        auto value = [&](int r, int s2) {
-            df_add2(Ah[r][s2], Al[r][s2], sh[r][s2], sl[r][s2]);
-            const float2 h = upk2(Ah[r][s2]), l = upk2(Al[r][s2]);
-            return df_to_double(h.x, l.x) + df_to_double(h.y, l.y);   // even + odd rows
-        };
-        int nblk = 0, s_hi = p_lo + share;
-        bool parked = false;
+        int nblk = 0;
         for (int p0 = p_lo; p0 < p_hi; p0 += GDF_SUB) {
             cp_async_wait_all();
             __syncthreads();   // this block's rows landed; every thread is done with the planes
@@ -383,57 +367,20 @@ __global__ void __launch_bounds__(GDF_MAXTHR, 2) gram_df_kernel(GramArgs a, long
                     }
                 nblk = 0;
             }
-            if (p0 + GDF_SUB >= s_hi && s_hi < p_hi) {
-                double* d = reinterpret_cast<double*>(smem_raw + park) + (size_t)tid * 4;
-#pragma unroll
-                for (int r = 0; r < 2; ++r)
-#pragma unroll
-                    for (int s2 = 0; s2 < 2; ++s2) {
-                        const double v = value(r, s2);
-                        d[2 * r + s2] = parked ? d[2 * r + s2] + v : v;
-                        sh[r][s2] = sl[r][s2] = Ah[r][s2] = Al[r][s2] = 0ull;
-                    }
-                parked = true;
-                nblk = 0;
-                s_hi += share;
-            }
         }
         cp_async_wait_all();   // the last (empty) group
         double acc[2][2];
-        {
-            const double* d = reinterpret_cast<const double*>(smem_raw + park) + (size_t)tid * 4;
 #pragma unroll
-            for (int r = 0; r < 2; ++r)
+        for (int r = 0; r < 2; ++r)
 #pragma unroll
-                for (int s2 = 0; s2 < 2; ++s2) {
-                    const double v = value(r, s2);
-                    acc[r][s2] = parked ? d[2 * r + s2] + v : v;
-                }
-        }
-        double* sacc = reinterpret_cast<double*>(smem_raw);
-        if (cl > 1) {
-            __syncthreads();   // the planes are read
-            if (active && rank > 0) {
-                double* d = sacc + (size_t)tid * 4;
-                d[0] = acc[0][0];
-                d[1] = acc[0][1];
-                d[2] = acc[1][0];
-                d[3] = acc[1][1];
+            for (int s2 = 0; s2 < 2; ++s2) {
+                df_add2(Ah[r][s2], Al[r][s2], sh[r][s2], sl[r][s2]);
+                const float2 h = upk2(Ah[r][s2]), l = upk2(Al[r][s2]);
+                acc[r][s2] = df_to_double(h.x, l.x) + df_to_double(h.y, l.y);   // even + odd rows
             }
-            gdf_cluster_sync();
-            if (active && rank == 0) {
-                for (int k = 1; k < cl; ++k) {
-                    const double* d = gdf_peer(sacc + (size_t)tid * 4, k);
-                    acc[0][0] += d[0];
-                    acc[0][1] += d[1];
-                    acc[1][0] += d[2];
-                    acc[1][1] += d[3];
-                }
-            }
-            gdf_cluster_sync();   // the others' memory is free again
-        }
         // groups > 0 hand their sums to group 0 through shared memory
-        if (P > 1 && rank == 0) {
+        double* sacc = reinterpret_cast<double*>(smem_raw);
+        if (P > 1) {
             __syncthreads();
             if (active && grp > 0) {
                 double* d = sacc + ((size_t)(grp - 1) * ntiles + (tid - grp * ntiles)) * 4;
@@ -452,6 +399,27 @@ __global__ void __launch_bounds__(GDF_MAXTHR, 2) gram_df_kernel(GramArgs a, long
                     acc[1][1] += d[3];
                 }
             }
+        }
+        if (cl > 1) {
+            __syncthreads();   // the group sums are read
+            if (active && grp == 0 && rank > 0) {
+                double* d = sacc + (size_t)tid * 4;
+                d[0] = acc[0][0];
+                d[1] = acc[0][1];
+                d[2] = acc[1][0];
+                d[3] = acc[1][1];
+            }
+            gdf_cluster_sync();
+            if (active && grp == 0 && rank == 0) {
+                for (int k = 1; k < cl; ++k) {
+                    const double* d = gdf_peer(sacc + (size_t)tid * 4, k);
+                    acc[0][0] += d[0];
+                    acc[0][1] += d[1];
+                    acc[1][0] += d[2];
+                    acc[1][1] += d[3];
+                }
+            }
+            gdf_cluster_sync();   // the others' memory is free again
         }
         if (active && grp == 0 && rank == 0) {
 #pragma unroll
@@ -524,23 +492,21 @@ cudaError_t launch_gram(const GramArgs& a, bool a_f32, bool b_f32, cudaStream_t 
             const int chunks = gram_chunks(a.Ng);
             const long long CH = gram_chunk_len(a.Ng);
             const void* fn = sub == 128 ? (const void*)gram_df_kernel<128> : (const void*)gram_df_kernel<64>;
-            const int park = (int)((smem + 15) / 16 * 16);   // the threads' sums over earlier shares
-            if (gdf_share((int)CH, sub) < CH) smem = park + (size_t)thr * 4 * sizeof(double);
             if (smem > 48 * 1024)
                 cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             // Few items leave one CTA an SM or less, which waits for its loads and its barriers in
-            // turn: clusters take the chunks' shares while all of them are resident (more chunks
-            // would lengthen the last CTA's sum over them).  The coarse update on 64^3 with 16
-            // columns, whose two Grams have one item each: 460 -> 429 us.
+            // turn: clusters of up to four CTAs share the chunks while all of them are resident
+            // (more chunks would lengthen the last CTA's sum over them).  The coarse update on 64^3
+            // with 16 columns, whose two Grams have one item each: 460 -> 429 us.
             int cl = 1, dev = 0, sms = 0, occ = 0;
             cudaError_t e = cudaGetDevice(&dev);
             if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             if (e != cudaSuccess) return e;
             const long long ctas = (long long)chunks * a.B;
-            if (ctas <= 2LL * sms && gdf_share((int)CH, sub) < CH) {
+            if (ctas <= 2LL * sms && CH >= 4 * sub) {
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, thr, smem);
                 if (e != cudaSuccess) return e;
-                if (GDF_SHARES * ctas <= (long long)occ * sms) cl = GDF_SHARES;
+                while (cl < 4 && (cl + 1) * ctas <= (long long)occ * sms) ++cl;
             }
             cudaLaunchConfig_t cfg{};
             cudaLaunchAttribute at[1];
@@ -553,7 +519,7 @@ cudaError_t launch_gram(const GramArgs& a, bool a_f32, bool b_f32, cudaStream_t 
             at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
             cfg.attrs = at;
             cfg.numAttrs = cl > 1 ? 1 : 0;
-            e = cudaLaunchKernelEx(&cfg, sub == 128 ? gram_df_kernel<128> : gram_df_kernel<64>, a, CH, chunks, cl, park);
+            e = cudaLaunchKernelEx(&cfg, sub == 128 ? gram_df_kernel<128> : gram_df_kernel<64>, a, CH, chunks, cl);
             if (e != cudaSuccess) return e;
             ++g_launch_count;
             return cudaGetLastError();
