@@ -427,7 +427,7 @@ cudaError_t gram_auto(pr_ctx* c, const GramArgs& ga, bool in_f32, bool k_exact) 
 
 pr_status pod_pipeline(pr_ctx* c, int B, int maxK, double gamma, double tau, bool in_f32, int cap,
                        int mmax, char* dest, size_t dest_bstride_elems, int* m_dest,
-                       bool ortho_blocks = false, bool k_exact = true) {
+                       bool ortho_blocks = false, bool k_exact = true, int items = 0) {
     const bool f32 = false;  // bases and their Grams are FP64
     cudaStream_t st = c->st;
     // Gram W^T W
@@ -439,6 +439,7 @@ pr_status pod_pipeline(pr_ctx* c, int B, int maxK, double gamma, double tau, boo
     ga.ldcols = c->ldcols;
     ga.Ng = c->Ng;
     ga.B = B;
+    ga.items = items > 0 ? items : c->N;
     ga.maxKA = maxK;
     ga.maxKB = maxK;
     ga.sym = true;
@@ -522,7 +523,7 @@ pr_status pod_pipeline(pr_ctx* c, int B, int maxK, double gamma, double tau, boo
 // 3 mmax^2 in Lo, R^T L R (steady flows) or the pieces R^T D R, R^T A0 R, R^T A1 R
 // (time-dependent flows, L(t) = D + c0(t) A0 + c1(t) A1, D = -eps Lap_h).
 pr_status galerkin(pr_ctx* c, char* R, size_t bstride_elems, const int* m, int B, int mmax, double* Mo,
-                   double* Lo, bool orthonormal = false) {
+                   double* Lo, bool orthonormal = false, int items = 0) {
     const bool f32 = false;
     pr_status s = cols_contig(c, R, bstride_elems * c->esz, m, 1, B, c->colsA, c->KA, c->esz);
     if (s != PR_OK) return s;
@@ -536,6 +537,7 @@ pr_status galerkin(pr_ctx* c, char* R, size_t bstride_elems, const int* m, int B
     ga.ldcols = c->ldcols;
     ga.Ng = c->Ng;
     ga.B = B;
+    ga.items = items > 0 ? items : c->N;
     ga.maxKA = mmax;
     ga.maxKB = mmax;
     ga.sym = true;
@@ -1133,11 +1135,11 @@ pr_status pr_iteration0(pr_ctx* c) {
     s = cols_contig(c, c->snap, 0, c->cnst + 1, 0, 1, c->colsA, c->KA, sizeof(double));
     if (s != PR_OK) return s;
     s = pod_pipeline(c, 1, c->ns0, c->gamma1, c->tau1, false, c->o.m_cap, c->mcap0, c->V0,
-                     (size_t)c->mcap0 * Ng, c->m0);
+                     (size_t)c->mcap0 * Ng, c->m0, false, true, 1);
     if (s != PR_OK) return s;
 
     // Galerkin matrices of V0 and projections of u_hat0, f
-    s = galerkin(c, c->V0, (size_t)c->mcap0 * Ng, c->m0, 1, c->mcap0, c->M0, c->L0);
+    s = galerkin(c, c->V0, (size_t)c->mcap0 * Ng, c->m0, 1, c->mcap0, c->M0, c->L0, false, 1);
     if (s != PR_OK) return s;
     {
         // p0 = V0^T u_hat0, q0 = V0^T f : gram of V0 columns against [u_hat0, f]
@@ -1151,7 +1153,7 @@ pr_status pr_iteration0(pr_ctx* c) {
         ga.KB = c->cnst + 3;  // 1 column
         ga.ldcols = 0;
         ga.Ng = Ng;
-        ga.B = 1;
+        ga.B = ga.items = 1;
         ga.maxKA = c->mcap0;
         ga.maxKB = 1;
         ga.part = c->gpart;
@@ -1875,6 +1877,7 @@ pr_status pr_op_gram(pr_ctx* c, const double* d_W, int n_cols, int B, double* d_
     ga.ldcols = c->ldcols;
     ga.Ng = c->Ng;
     ga.B = B;
+    ga.items = c->N;
     ga.maxKA = n_cols;
     ga.maxKB = n_cols;
     ga.sym = true;
@@ -1900,7 +1903,7 @@ pr_status pr_op_coarse_update(pr_ctx* c, const void* d_R, int m, const double* d
     double* Mr = c->Mr + (size_t)c->N * c->mcap2 * c->mcap2;
     double* Lr = c->Lr + (size_t)c->N * 3 * c->mcap2 * c->mcap2;
     if (m > 0) {
-        s = galerkin(c, (char*)d_R, (size_t)c->mcap2 * c->Ng, c->m2 + c->N, 1, c->mcap2, Mr, Lr);
+        s = galerkin(c, (char*)d_R, (size_t)c->mcap2 * c->Ng, c->m2 + c->N, 1, c->mcap2, Mr, Lr, false, 1);
         if (s != PR_OK) return s;
     }
     CoarseSweepArgs a = coarse_args(c);

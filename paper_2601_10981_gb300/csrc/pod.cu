@@ -497,12 +497,13 @@ cudaError_t launch_gram(const GramArgs& a, bool a_f32, bool b_f32, cudaStream_t 
             // Few items leave one CTA an SM or less, which waits for its loads and its barriers in
             // turn: clusters of up to four CTAs share the chunks while all of them are resident
             // (more chunks would lengthen the last CTA's sum over them).  The coarse update on 64^3
-            // with 16 columns, whose two Grams have one item each: 460 -> 429 us.
+            // with 16 columns, whose two Grams have one item each: 460 -> 429 us.  The cluster's size
+            // orders the sums, so it follows the caller's `items` and not B.
             int cl = 1, dev = 0, sms = 0, occ = 0;
             cudaError_t e = cudaGetDevice(&dev);
             if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             if (e != cudaSuccess) return e;
-            const long long ctas = (long long)chunks * a.B;
+            const long long ctas = (long long)chunks * std::max(1, a.items);
             if (ctas <= 2LL * sms && CH >= 4 * sub) {
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, thr, smem);
                 if (e != cudaSuccess) return e;

@@ -256,6 +256,8 @@ struct GramArgs {
     int ldcols;
     long long Ng;
     int B;
+    int items;                // the items that the order of the sums is chosen for, whatever B: the
+                              // context's, or 1 (an item then gets the same Gram in every call)
     int maxKA, maxKB;
     bool sym;
     double* part;             // [B][chunks][maxKA*maxKB]

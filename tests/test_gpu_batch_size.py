@@ -1,0 +1,44 @@
+"""An item's POD does not depend on how many items share the call: wave mode and requests that
+are run together give the bits of the single launch (for a fixed group_ctas)."""
+import numpy as np
+import pytest
+
+import pr_inputs as pi
+from test_gpu_gram_tc import _columns
+
+pytestmark = pytest.mark.gpu
+
+
+def same_alone_and_together(fn, Wt):
+    """fn on all items, and on each of the first and last alone and the first two together."""
+    whole = fn(Wt)
+    B = Wt.shape[0]
+    for lo, hi in [(0, 1), (0, 2), (B - 1, B)]:
+        part = fn(Wt[lo:hi].contiguous())
+        for x, y in zip(whole, part):
+            assert np.array_equal(x[lo:hi], y), (lo, hi)
+
+
+# chunks of one share and of three, ragged ones, several groups of rows a CTA and one
+@pytest.mark.parametrize("n,K,B", [(64, 16, 5), (45, 40, 6), (41, 3, 9), (37, 33, 4), (64, 60, 3)])
+def test_double_float_gram(gpu, n, K, B):
+    bd, torch = gpu
+    w = pi.Workload("gram", n, pi.Flow("abc"), 0.05, 1.0, B, 1e-3, n_snap=64, m_cap=32)
+    s = bd.Parareal.from_workload(w, precision=bd.PR_FP32)
+    Wt = torch.from_numpy(np.ascontiguousarray(_columns(n, K, B, seed=n * K))).to("cuda")
+    same_alone_and_together(lambda x: [s.op_gram(x, tensor=False, df=True).cpu().numpy()], Wt)
+    s.close()
+
+
+# contexts of one or two items, whose chunks are shared by clusters
+@pytest.mark.parametrize("n,K,B", [(41, 3, 1), (47, 17, 2), (45, 33, 1), (64, 16, 1), (41, 60, 1)])
+def test_double_float_gram_in_clusters(gpu, n, K, B):
+    bd, torch = gpu
+    w = pi.Workload("gram", n, pi.Flow("abc"), 0.05, 1.0, B, 1e-3, n_snap=64, m_cap=32)
+    s = bd.Parareal.from_workload(w, precision=bd.PR_FP32)
+    Wt = torch.from_numpy(np.ascontiguousarray(_columns(n, K, B, seed=n + K))).to("cuda")
+    Gd = s.op_gram(Wt, tensor=False, df=True).cpu().numpy()
+    G64 = s.op_gram(Wt, tensor=False).cpu().numpy()
+    s.close()
+    for b in range(B):   # the bound of the double-float Gram on smaller grids
+        assert np.abs(Gd[b] - G64[b]).max() < 1e-14 * np.abs(G64[b]).max()
