@@ -153,7 +153,7 @@ enum pr_method { PR_METHOD_ADAPTIVE = 0, PR_METHOD_PARAREAL_I = 1, PR_METHOD_PAR
  * data; FP64 beyond).  PR_GRAM_TENSOR: the tensor cores, with the values cut into
  * error-free BF16 digits (FP64-accurate, see pr_op_gram; up to 64 columns, double-float
  * beyond).  PR_GRAM_AUTO: the tensor cores for snapshot windows of 20..32 and 55..64
- * columns, and of 33..54 where a call has 262144 points or more (and the context's
+ * columns, and of 33..54 where n_sub n^3 is 262144 or more (and the context's
  * spin_limit is 4096 or more: double-float waits for nothing), where they are faster;
  * double-float otherwise (and for the Cholesky-QR Grams,
  * whose column counts are POD dimensions known only on the device).  The FP64 mode always
@@ -349,10 +349,9 @@ pr_status pr_op_pod(pr_ctx* ctx, const void* d_W, int w_f32, int n_cols, int B, 
  *   1: the tensor cores (tcgen05.mma, BF16 operands, FP32 accumulation; n_cols <= 64).
  *      Each column is aligned to its largest magnitude and each value truncated to 56
  *      bits and cut into eight balanced base-128 integer digits, which BF16 holds
- *      exactly; digit products are summed exactly in FP32 over windows of points.  Up to
- *      32 columns the windows are folded into 128-bit integers, so the result is the
- *      digit sum rounded once to FP64 (bit-reproducible); 33..64 columns fold them into
- *      FP64 every 1024 points.  Either way FP64-accurate.
+ *      exactly; digit products are summed exactly in FP32 over windows of points and
+ *      these in integers, so the result is the digit sum rounded once to FP64
+ *      (bit-reproducible, whatever B): FP64-accurate.
  *   2: double-float arithmetic on the FP32 pipe (the FP32 mode's default kernel).
  *   0: FP64 arithmetic.
  * B <= n_sub + 1, n_cols <= the context's largest POD window.  Synchronises. */

@@ -400,9 +400,9 @@ pr_status cols_contig(pr_ctx* c, const char* base, size_t bstride_bytes, const i
 // ortho_blocks: the snapshot columns are blocks of orthonormal bases (c->colblk says
 // which); the FP32 mode then takes their diagonal Gram blocks as the identity.
 // Symmetric Grams of the FP32 mode: on the tensor cores (error-free BF16 digit products,
-// FP64-accurate; gram_tc.cu) for windows of 20..64 columns (gram_mode PR_GRAM_AUTO), for every
-// width up to 64 (PR_GRAM_TENSOR), or never
-// (PR_GRAM_DF); every other Gram runs in double-float or FP64.
+// FP64-accurate; gram_tc.cu) for windows of 20..32 and 55..64 columns and, in contexts whose windows
+// hold 262,144 points or more, of 33..54 (gram_mode PR_GRAM_AUTO), for every width up to 64 (PR_GRAM_TENSOR), or
+// never (PR_GRAM_DF); every other Gram runs in double-float or FP64.
 // k_exact: every item has maxKA columns (a snapshot window), not a cap on a POD dimension
 // that lives on the device; the automatic choice of the tensor cores needs the column
 // count (a Gram of 4 columns under a cap of 32 is faster in double-float).
@@ -416,10 +416,12 @@ cudaError_t gram_auto(pr_ctx* c, const GramArgs& ga, bool in_f32, bool k_exact) 
     // (33..64) from 262,144 points in all (op_gram, 33 and 54 columns: 64^3 x 16 1.07 vs 1.81
     // and 1.22 vs 4.07 ms, 32^3 x 16 0.23 vs 0.30 and 0.27 vs 0.66, 64^3 x 1 0.19 vs 0.21 and
     // 0.28 vs 0.39; 32^3 x 1 0.13 vs 0.09 and 0.19 vs 0.14), and beyond the double-float
-    // kernel's 384 output tiles a pass (55 columns) always.  Double-float waits for nothing: a
-    // context whose waits may not last (spin_limit below a few milliseconds) keeps it there.
+    // kernel's 384 output tiles a pass (55 columns) always.  The points are those of the context's N
+    // items, not of the call's: waves and the single launch take the same kernel.
+    // Double-float waits for nothing: a context whose waits may not last (spin_limit below a few
+    // milliseconds) keeps it there.
     const bool narrow = ga.maxKA >= 20 && ga.maxKA <= 32;
-    const bool wide = ga.maxKA > 54 || (ga.maxKA > 32 && ga.B * ga.Ng >= 262144 && c->o.spin_limit >= 4096);
+    const bool wide = ga.maxKA > 54 || (ga.maxKA > 32 && ga.items * ga.Ng >= 262144 && c->o.spin_limit >= 4096);
     if (fits && (mode == PR_GRAM_TENSOR || (mode == PR_GRAM_AUTO && k_exact && (narrow || wide))))
         return launch_gram_tc(ga, c->colmax, gram_tc_max_cols(), c->derr, c->o.spin_limit, c->st);
     return launch_gram(ga, in_f32, in_f32, c->st);
