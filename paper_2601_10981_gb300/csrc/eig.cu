@@ -89,8 +89,7 @@ __device__ __forceinline__ void eig_angle(double app, double apq, double aqq, do
 
 __host__ __device__ __forceinline__ size_t eig_doubles(int Kp, int C) {
     const int np = Kp / 2, nsl = (np + C - 1) / C, nv = (Kp + C - 1) / C;
-    return (size_t)4 * nsl * Kp + (size_t)(nv * (Kp + 1) + 1) / 2 * 2 + 4 * np + 6 * np + 2 * Kp +
-           2 * EIG_MAXC * EIG_WARPS;
+    return (size_t)4 * nsl * Kp + (size_t)(nv * (Kp + 1) + 1) / 2 * 2 + 4 * np + 6 * np + 4 * Kp;
 }
 static size_t eig_smem(int Kp, int C) { return eig_doubles(Kp, C) * sizeof(double) + (size_t)Kp * sizeof(int); }
 
@@ -115,8 +114,8 @@ __global__ void __launch_bounds__(EIG_THREADS) eig_pod_kernel(EigArgs a, int C) 
     double* nd = reinterpret_cast<double*>(cs + 2 * np);   // [2][np][3]: a_pp, a_pq, a_qq
     double* lam = nd + 6 * np;                          // [Kp]
     double* sq = lam + Kp;                              // [Kp]
-    double* red = sq + Kp;                              // [EIG_MAXC][EIG_WARPS][2]
-    int* perm = reinterpret_cast<int*>(red + 2 * EIG_MAXC * EIG_WARPS);   // [Kp]
+    double* red = sq + Kp;                              // [Kp][2]: a row's off-diagonal and diagonal squares
+    int* perm = reinterpret_cast<int*>(red + 2 * Kp);   // [Kp]
     __shared__ int s_stop, s_e, s_r, s_m;
     const double* Gb = a.G + (size_t)b * a.ldG_b;
 
@@ -190,26 +189,28 @@ __global__ void __launch_bounds__(EIG_THREADS) eig_pod_kernel(EigArgs a, int C) 
         // convergence: off-diagonal Frobenius norm against the whole matrix
         {
             const double* A = A0 + (size_t)cur * 2 * nsl * Kp;
-            double off = 0.0, dia = 0.0;
-            for (int e = tid; e < 2 * ns * Kp; e += EIG_THREADS) {
-                const int lr = e / Kp, pc = e - lr * Kp;
-                const double v = A[e];
-                if (2 * s0 + lr == pc) dia = fma(v, v, dia);
-                else off = fma(v, v, off);
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                off += __shfl_xor_sync(0xffffffffu, off, o);
-                dia += __shfl_xor_sync(0xffffffffu, dia, o);
-            }
-            if (lane < C) {
-                double* r = C > 1 ? eig_peer(red, lane) : red;
-                r[2 * (rank * EIG_WARPS + warp)] = off;
-                r[2 * (rank * EIG_WARPS + warp) + 1] = dia;
+            // row by row, eight lanes a row, then the rows in a fixed order: the same sums, and so
+            // the same rotations, for every C (which follows the number of matrices in the launch)
+            for (int l0 = 0; l0 < 2 * ns; l0 += EIG_THREADS / 8) {
+                const int lr = l0 + (tid >> 3), pr = 2 * s0 + lr;
+                double off = 0.0;
+                if (lr < 2 * ns)
+                    for (int pc = tid & 7; pc < Kp; pc += 8) {
+                        const double v = A[lr * Kp + pc];
+                        if (pc != pr) off = fma(v, v, off);
+                    }
+                for (int o = 4; o > 0; o >>= 1) off += __shfl_xor_sync(0xffffffffu, off, o);
+                if (lr < 2 * ns && (tid & 7) < C) {
+                    const double v = A[lr * Kp + pr];
+                    double* r = C > 1 ? eig_peer(red, tid & 7) : red;
+                    r[2 * pr] = off;
+                    r[2 * pr + 1] = v * v;
+                }
             }
             cluster_sync();
             if (warp == 0) {
-                off = dia = 0.0;
-                for (int i = lane; i < C * EIG_WARPS; i += 32) {
+                double off = 0.0, dia = 0.0;
+                for (int i = lane; i < Kp; i += 32) {
                     off += red[2 * i];
                     dia += red[2 * i + 1];
                 }

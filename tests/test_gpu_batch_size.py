@@ -5,6 +5,7 @@ import pytest
 
 import pr_inputs as pi
 from test_gpu_gram_tc import _columns
+from test_gpu_waves import _iterates
 
 pytestmark = pytest.mark.gpu
 
@@ -69,3 +70,41 @@ def test_pod_of_middle_widths(gpu, n, K, B):
 
     same_alone_and_together(pod, Wt)
     s.close()
+
+
+# the eigensolver's cluster of CTAs follows the number of matrices: 1, 2, 4 and 8 of them
+@pytest.mark.parametrize("K,B", [(64, 20), (34, 40), (17, 80), (71, 30)])
+def test_eigensolver(gpu, K, B):
+    bd, torch = gpu
+    n, cap = 6, min(K, 32)
+    w = pi.Workload("eig", n, pi.Flow("abc"), 0.05, 1.0, B, 1.0 / (B * (K - 1)), n_snap=K, m_cap=cap)
+    s = bd.Parareal.from_workload(w, precision=bd.PR_FP64)
+    rng = np.random.default_rng(K)
+    W = np.stack([(np.linalg.qr(rng.standard_normal((n ** 3, K)))[0] * np.logspace(0, -5, K)) @
+                  np.linalg.qr(rng.standard_normal((K, K)))[0] for _ in range(B)])
+    Wt = torch.from_numpy(np.ascontiguousarray(np.swapaxes(W, 1, 2))).cuda().reshape(B, K, n, n, n)
+
+    def pod(x):
+        R, m = s.op_pod(x, 1.0, cap)
+        return [R.cpu().numpy(), m]
+
+    same_alone_and_together(pod, Wt)
+    s.close()
+
+
+# waves whose last one holds one or two windows, against the single launch
+@pytest.mark.parametrize("precision,n,N,ns,wave", [(1, 45, 7, 40, 3), (0, 45, 5, 12, 2), (1, 64, 5, 64, 2), (1, 64, 4, 40, 3)])
+def test_wave_form(gpu, precision, n, N, ns, wave):
+    bd, torch = gpu
+    dt = 1e-3
+    w = pi.Workload("waves", n, pi.Flow("kolmogorov", k=2), 0.02, N * (ns - 1) * dt, N, dt, n_snap=ns, m_cap=16, f_seed=3)
+    s1, U1 = _iterates(bd, w, N, precision, group_ctas=9)
+    m1 = s1.diagnostics()
+    s1.close()
+    s2, U2 = _iterates(bd, w, N, precision, group_ctas=9, wave=wave)
+    m2 = s2.diagnostics()
+    s2.close()
+    for k in range(N + 1):
+        assert np.array_equal(U1[k], U2[k]), (k, float(np.max(np.abs(U1[k] - U2[k]))))
+    # the subintervals of the last iteration (older entries are an earlier iteration's)
+    assert np.array_equal(m1["m1"][N - 1:], m2["m1"][N - 1:]) and np.array_equal(m1["m2"][N:], m2["m2"][N:])
