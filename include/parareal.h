@@ -349,9 +349,11 @@ pr_status pr_op_pod(pr_ctx* ctx, const void* d_W, int w_f32, int n_cols, int B, 
  *   1: the tensor cores (tcgen05.mma, BF16 operands, FP32 accumulation; n_cols <= 64).
  *      Each column is aligned to its largest magnitude and each value truncated to 56
  *      bits and cut into eight balanced base-128 integer digits, which BF16 holds
- *      exactly; digit products are summed exactly in FP32 over windows of points and
- *      these in integers, so the result is the digit sum rounded once to FP64
- *      (bit-reproducible, whatever B): FP64-accurate.
+ *      exactly; digit products are summed exactly in FP32 over windows of points.  Up to
+ *      32 columns the windows are folded into 128-bit integers, so the result is the
+ *      digit sum rounded once to FP64 (bit-reproducible); 33..64 columns sum exactly over a
+ *      chunk of points, rounded once (the chunks follow n_sub, not B).  Either way
+ *      FP64-accurate.
  *   2: double-float arithmetic on the FP32 pipe (the FP32 mode's default kernel).
  *   0: FP64 arithmetic.
  * B <= n_sub + 1, n_cols <= the context's largest POD window.  Synchronises. */

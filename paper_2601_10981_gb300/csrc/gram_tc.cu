@@ -21,10 +21,9 @@
 // those with s + t = c + 1, from at most four (s, t) pairs each.  Every 1024 points
 // (4 x 1024 x 2^12 = 2^24) the eight tiles (c = 2..9, all pairs with s + t <= 9; the
 // dropped ones weigh below 2^-58 of a leading product) are read back with tcgen05.ld and
-// added, with their weights, into exact 96-bit integers; their sums over the chunks are exact
-// too and rounded once.  The only other rounding is the 56-bit truncation of each value, so the
-// result has the accuracy of an FP64 Gram, and does not depend on how the points are cut into
-// chunks (whose number follows the number of items in the launch).
+// added, with their weights, into exact 96-bit integers, which are rounded once a chunk.
+// The only other rounding is the 56-bit truncation of each value, so the result has the
+// accuracy of an FP64 Gram.
 //
 // Two forms share the digit scheme: the wide one described here (up to 64 columns,
 // gram_tc_kernel) and a narrow, warp-specialised one for up to 32 columns
@@ -845,23 +844,14 @@ __global__ void __launch_bounds__(640, 1) gram_tc_kernel(GramArgs a, int CH, int
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         mbar_arrive(tempty);   // the tiles may be overwritten
         if (!plast) return;
-        // ---- the unit's partial: 2^7 top + bottom (64 rows, two warps on), exact; the upper
-        // triangle, row by row.  The only unit of an item writes G itself.
+        // ---- the unit's partial: 2^7 top + bottom (64 rows, two warps on), rounded once
         tc_prod_sync();
         const int b = pu / chunks, chunk = pu - b * chunks;
         const int K = a.KA[b];
-        const int mk = a.maxKA;
-        const size_t outsz = (size_t)mk * (mk + 1) / 2;
-        auto at = [&](int i, int j) { return (size_t)(i * mk - i * (i - 1) / 2 + (j - i)); };
-        __int128* bpart = reinterpret_cast<__int128*>(a.part) + (size_t)b * chunks * outsz;
-        double* Gb = a.G + (size_t)b * a.ldG_b;
-        auto put = [&](int i, int j, __int128 S) {
-            const double g = i128_to_double(
-                S, col_exp(colmax[(size_t)b * ld + i]) + col_exp(colmax[(size_t)b * ld + j]) - 70);
-            Gb[(size_t)i * a.ldG + j] = g;
-            Gb[(size_t)j * a.ldG + i] = g;
-        };
+        const size_t outsz = (size_t)a.maxKA * a.maxKB;
+        double* mypart = a.part + ((size_t)b * chunks + chunk) * outsz;
         if (top && irow < K) {
+            const int ei = col_exp(colmax[(size_t)b * ld + irow]);
 #pragma unroll 1
             for (int j = 0; j < 16; ++j) {
                 const int jj = 16 * cq + j;
@@ -871,16 +861,11 @@ __global__ void __launch_bounds__(640, 1) gram_tc_kernel(GramArgs a, int CH, int
                     return ((__int128)(int)v[2 * TC_PROD + o] << 64) |
                            ((unsigned long long)v[TC_PROD + o] << 32 | v[o]);
                 };
-                const __int128 S = (word(0) << 7) + word(64);
-                if (chunks == 1) put(irow, jj, S);
-                else bpart[chunk * outsz + at(irow, jj)] = S;
+                mypart[(size_t)irow * a.maxKB + jj] =
+                    i128_to_double((word(0) << 7) + word(64), ei + col_exp(colmax[(size_t)b * ld + jj]) - 70);
             }
         }
-        if (chunks == 1) {
-            tc_prod_sync();   // the sums are read
-            return;
-        }
-        // the last unit of item b adds the partials
+        // the last unit of item b sums the chunk partials in chunk order
         __threadfence();
         tc_prod_sync();
         if (tid == 0) {
@@ -890,21 +875,25 @@ __global__ void __launch_bounds__(640, 1) gram_tc_kernel(GramArgs a, int CH, int
         tc_prod_sync();
         if (s_last) {
             __threadfence();
+            const double* bpart = a.part + (size_t)b * chunks * outsz;
+            double* Gb = a.G + (size_t)b * a.ldG_b;
             for (int o = tid; o < K * K; o += TC_PROD) {
                 const int i = o / K, j = o - i * K;
                 if (j < i) continue;
-                const __int128* src = bpart + at(i, j);   // loads in batches of 4 independent ones
-                __int128 S = 0;
+                // chunk order (reproducible), loads in batches of 8 independent ones
+                const double* src = bpart + (size_t)i * a.maxKB + j;
+                double sum = 0.0;
                 int cc = 0;
-                for (; cc + 4 <= chunks; cc += 4) {
-                    __int128 v[4];
+                for (; cc + 8 <= chunks; cc += 8) {
+                    double v[8];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) v[e] = src[(size_t)(cc + e) * outsz];
+                    for (int e = 0; e < 8; ++e) v[e] = src[(size_t)(cc + e) * outsz];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) S += v[e];
+                    for (int e = 0; e < 8; ++e) sum += v[e];
                 }
-                for (; cc < chunks; ++cc) S += src[(size_t)cc * outsz];
-                put(i, j, S);
+                for (; cc < chunks; ++cc) sum += src[(size_t)cc * outsz];
+                Gb[(size_t)i * a.ldG + j] = sum;
+                Gb[(size_t)j * a.ldG + i] = sum;
             }
             if (tid == 0) st_relaxed_u32(a.counter + b, 0u);
         }
@@ -994,12 +983,14 @@ cudaError_t launch_gram_tc(const GramArgs& a, unsigned long long* colmax, int ld
     // (short units pay a read-back, the partials' fences and the last CTA's sum over them: 16
     // windows of 33 columns on 32^3, 791 us in units of 320 points, 230 us in one wave; 16 of 54
     // on 64^3, 2.64 and 1.22 ms)
-    const long long waves = std::max<long long>(1, a.B * a.Ng / 16384 / std::max(1, sms));
-    const int cw = (int)std::min<long long>(chunks, std::max<long long>(1, waves * sms / a.B));
+    auto units = [&](long long items) {
+        const long long waves = std::max<long long>(1, items * a.Ng / 16384 / std::max(1, sms));
+        return (int)std::min<long long>(chunks, std::max<long long>(1, waves * sms / items));
+    };
     if (a.maxKA <= N2_COLS && chunks >= 2) {
         // narrow form: at most one unit for two partial slots of the other Gram kernels, since a
         // unit's partial is K x K 128-bit integers
-        const int ctc = std::min(cw, chunks / 2);
+        const int ctc = std::min(units(a.B), chunks / 2);
         const long long U2 = ((a.Ng + ctc - 1) / ctc + N2_PTS - 1) / N2_PTS * N2_PTS;
         const int chunks2 = (int)((a.Ng + U2 - 1) / U2);
         e = cudaFuncSetAttribute((const void*)gram_tc32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1010,10 +1001,13 @@ cudaError_t launch_gram_tc(const GramArgs& a, unsigned long long* colmax, int ld
         ++g_launch_count;
         return cudaGetLastError();
     }
-    // wide form, one CTA an SM (the tiles take all 512 tensor-memory columns); a unit's partial is the
-    // upper triangle in 128-bit integers, K (K + 1) doubles' room where the other kernels' slots have K^2
-    const int cx = std::min(cw, std::max(1, (int)((long long)chunks * a.maxKA / (a.maxKA + 1))));
-    const int CHw = (int)(((a.Ng + cx - 1) / cx + TC_PTS - 1) / TC_PTS * TC_PTS);
+    // wide form, one CTA an SM (the tiles take all 512 tensor-memory columns).  It rounds a unit's
+    // sums, and an item's Gram may not depend on how many items share the call: units of the context's
+    // items.  (Exact 128-bit partials, rounded at the end, would allow any units, but Grams of windows
+    // with fewer modes than columns, so rounded, take the Jacobi iteration more sweeps: four windows
+    // of 64 on 128^3, 13.8 -> 15.4 ms a POD call.)
+    const int cw = units(std::max(1, a.items));
+    const int CHw = (int)(((a.Ng + cw - 1) / cw + TC_PTS - 1) / TC_PTS * TC_PTS);
     const int chunksw = (int)((a.Ng + CHw - 1) / CHw);
     e = cudaFuncSetAttribute((const void*)gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
     if (e != cudaSuccess) return e;
