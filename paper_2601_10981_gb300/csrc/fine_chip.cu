@@ -58,7 +58,7 @@ struct ChipShared {
     KT red[CHIP_MAXQ * CHIP_MAXWARPS];
     double slot[2][CHIP_MAXQ][CHIP_MAXC];   // partials of all CTAs, alternating
     double tot[8];
-    double rho, inv_rv, thr, thr2;
+    double rho, inv_rv, iom, thr, thr2;
     KT al, om, be;   // alpha, omega, beta for the vector updates (rounded once a CTA)
     int safe, act, status;
 };
@@ -71,7 +71,11 @@ __device__ __forceinline__ bool chip_zero(double x) { return (__double_as_longlo
 __device__ __forceinline__ bool chip_le(double a, double b) { return __double_as_longlong(a) <= __double_as_longlong(b); }
 
 // What follows a stopping test.
-enum ChipAct { CHIP_GO = 0, CHIP_FULL = 1, CHIP_HALF = 2, CHIP_KEEP = 3 };
+enum ChipAct { CHIP_GO = 0, CHIP_FULL = 1, CHIP_HALF = 2, CHIP_KEEP = 3, CHIP_CHECK = 4 };
+// ||r||^2 = <s,s> - omega <t,s> below 2^-17 of <s,s> is not trusted in the FP32 mode, whose sums hold
+// about 2^-20: unless even that would meet the threshold, r is formed and summed (CHIP_CHECK).  It
+// happens where half a step cuts the residual several hundredfold, as on a first step from rest.
+constexpr unsigned CHIP_CANCEL = 17;
 
 __device__ __forceinline__ void chip_cluster_sync() {
     asm volatile("barrier.cluster.arrive.release;" ::: "memory");
@@ -512,6 +516,22 @@ __global__ void __launch_bounds__(512, 1) fine_chip_kernel(FineArgs a, ChipPlan 
                         }
                     }
                     __syncthreads();
+                    // what follows from ||r||^2 and <rhat, r>; beta and rho if another iteration does
+                    auto after = [&](double rr1, double rho_new, double iom) -> int {
+                        if (!chip_finite(rr1)) {
+                            sh.status = DERR_NONFINITE;
+                        } else if (met(rr1)) {
+                        } else if (chip_zero(rho_new)) {
+                            sh.status = DERR_BREAKDOWN;
+                        } else if (it >= J.maxit) {
+                            sh.status = DERR_NOT_CONVERGED;
+                        } else {
+                            sh.be = (KT)(rho_new * iom * sh.inv_rv);   // (rho'/rho)(alpha/omega)
+                            sh.rho = rho_new;
+                            return CHIP_GO;
+                        }
+                        return CHIP_FULL;
+                    };
                     KT acc[5] = {};
                     stencil(R, [&](int o, int z, int y, int x0, const Nb7<KT, W>& q) {
                         const Vec<KT, W> tv = applyA(o, z, y, x0, q);
@@ -552,20 +572,11 @@ __global__ void __launch_bounds__(512, 1) fine_chip_kernel(FineArgs a, ChipPlan 
                                 } else {
                                     const double rr1 = fma(-om, ts, ss);                    // ||s - omega t||^2
                                     const double rho_new = fma(-om, sh.tot[3], sh.tot[4]);   // <rhat, r>
-                                    if (!chip_finite(rr1)) {
-                                        sh.status = DERR_NONFINITE;
-                                        act2 = CHIP_FULL;
-                                    } else if (met(rr1)) {
-                                        act2 = CHIP_FULL;
-                                    } else if (chip_zero(rho_new)) {
-                                        sh.status = DERR_BREAKDOWN;
-                                        act2 = CHIP_FULL;
-                                    } else if (it >= J.maxit) {
-                                        sh.status = DERR_NOT_CONVERGED;
-                                        act2 = CHIP_FULL;
+                                    if (DF && chip_finite(rr1) && chip_exp(rr1) + CHIP_CANCEL < chip_exp(ss)) {
+                                        act2 = met(0x1p-17 * ss) ? CHIP_FULL : CHIP_CHECK;
+                                        sh.iom = iom;
                                     } else {
-                                        sh.be = (KT)(rho_new * iom * sh.inv_rv);   // (rho'/rho)(alpha/omega)
-                                        sh.rho = rho_new;
+                                        act2 = after(rr1, rho_new, iom);
                                     }
                                 }
                             }
@@ -573,6 +584,23 @@ __global__ void __launch_bounds__(512, 1) fine_chip_kernel(FineArgs a, ChipPlan 
                             sh.act = act2;
                         }
                     });
+                    if (DF && sh.act == CHIP_CHECK) {
+                        const KT om = sh.om;
+                        KT chk[2] = {(KT)0, (KT)0};
+                        for (int o = tid * W; o < npl * n2; o += nthr * W) {
+                            const Vec<KT, W> sv = vload<KT, W>(R + own + o), tv = vload<KT, W>(T + own + o);
+                            const Vec<KT, W> hv = vload<KT, W>(first ? P + own + o : RH + o);
+#pragma unroll
+                            for (int e = 0; e < W; ++e) {
+                                const KT rn = sv.v[e] - om * tv.v[e];
+                                chk[0] += rn * rn;
+                                chk[1] += hv.v[e] * rn;
+                            }
+                        }
+                        reduce(chk, [&]() {
+                            if (lane == 0) sh.act = after(sh.tot[0], sh.tot[1], sh.iom);
+                        });
+                    }
                 }
                 act = sh.act;
                 if (act != CHIP_GO) break;
