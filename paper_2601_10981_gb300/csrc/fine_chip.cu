@@ -270,16 +270,13 @@ __global__ void __launch_bounds__(512, 1) fine_chip_kernel(FineArgs a, ChipPlan 
     };
 
     chip_cluster_sync();   // every CTA of the cluster runs: its shared memory may be written
-    // The products of the second half of an iteration.  <rhat, s> = rho - alpha <rhat, v> is zero
-    // by the choice of alpha, but only as far as rho is <rhat, r>: taken as zero, rho keeps the rounding
-    // of the first iteration while <rhat, r> falls with the residual, and the FP64 mode no longer
-    // converged from about nine iterations a step on.
-    auto dots2 = [](KT (&s)[5], KT tv, KT sv, KT hv) {
+    // The products of the second half of an iteration, <rhat, s> with NQ = 5 (FINE_EARLY)
+    auto dots2 = [](auto& s, KT tv, KT sv, KT hv) {
         s[0] += tv * sv;
         s[1] += tv * tv;
         s[2] += sv * sv;
         s[3] += hv * tv;
-        s[4] += hv * sv;
+        if constexpr (sizeof(s) / sizeof(s[0]) == 5) s[4] += hv * sv;
     };
     for (int b = cl; b < a.B; b += gridDim.x / C) {
         int jb = 0, lb = b;
@@ -532,58 +529,67 @@ __global__ void __launch_bounds__(512, 1) fine_chip_kernel(FineArgs a, ChipPlan 
                         }
                         return CHIP_FULL;
                     };
-                    KT acc[5] = {};
-                    stencil(R, [&](int o, int z, int y, int x0, const Nb7<KT, W>& q) {
-                        const Vec<KT, W> tv = applyA(o, z, y, x0, q);
-                        vstore(T + own + o, tv);
-                        push(Tb, Ta, o, tv);
-                        const Vec<KT, W> hv = vload<KT, W>(first ? P + own + o : RH + o);
-                        KT s[5] = {};
-#pragma unroll
-                        for (int e = 0; e < W; ++e) {
-                            if constexpr (W == 1) {
-                                dots2(acc, tv.v[e], q.c.v[e], hv.v[e]);
-                            } else {
-                                dots2(s, tv.v[e], q.c.v[e], hv.v[e]);
-                            }
-                        }
-                        if constexpr (W > 1) {
-#pragma unroll
-                            for (int k = 0; k < 5; ++k) acc[k] += s[k];
-                        }
-                    });
-                    reduce(acc, [&]() {
-                        const double ts = sh.tot[0], tt = sh.tot[1], ss = sh.tot[2];
-                        const double qv = (lane == 0 ? ts : tt) / (lane == 0 ? tt : ts);   // omega, 1 / omega
-                        const double iom = __shfl_sync(0xffffffffu, qv, 1);
-                        if (lane == 0) {
-                            int act2 = CHIP_GO;
-                            double om = 0.0;
-                            if (chip_finite(ss) && met(ss)) {
-                                act2 = CHIP_HALF;
-                            } else if (chip_zero(tt) || !chip_finite(tt)) {
-                                sh.status = chip_finite(tt) ? DERR_BREAKDOWN : DERR_NONFINITE;
-                                act2 = CHIP_HALF;
-                            } else {
-                                om = qv;
-                                if (chip_zero(om)) sh.status = DERR_BREAKDOWN;
-                                if (sh.status != 0) {
-                                    act2 = CHIP_HALF;
+                    auto half = [&](auto& acc) {
+                        constexpr int NQ = sizeof(acc) / sizeof(acc[0]);
+                        stencil(R, [&](int o, int z, int y, int x0, const Nb7<KT, W>& q) {
+                            const Vec<KT, W> tv = applyA(o, z, y, x0, q);
+                            vstore(T + own + o, tv);
+                            push(Tb, Ta, o, tv);
+                            const Vec<KT, W> hv = vload<KT, W>(first ? P + own + o : RH + o);
+                            [[maybe_unused]] KT s[NQ] = {};
+    #pragma unroll
+                            for (int e = 0; e < W; ++e) {
+                                if constexpr (W == 1) {
+                                    dots2(acc, tv.v[e], q.c.v[e], hv.v[e]);
                                 } else {
-                                    const double rr1 = fma(-om, ts, ss);                    // ||s - omega t||^2
-                                    const double rho_new = fma(-om, sh.tot[3], sh.tot[4]);   // <rhat, r>
-                                    if (DF && chip_finite(rr1) && chip_exp(rr1) + CHIP_CANCEL < chip_exp(ss)) {
-                                        act2 = met(0x1p-17 * ss) ? CHIP_FULL : CHIP_CHECK;
-                                        sh.iom = iom;
-                                    } else {
-                                        act2 = after(rr1, rho_new, iom);
-                                    }
+                                    dots2(s, tv.v[e], q.c.v[e], hv.v[e]);
                                 }
                             }
-                            sh.om = (KT)om;
-                            sh.act = act2;
-                        }
-                    });
+                            if constexpr (W > 1) {
+    #pragma unroll
+                                for (int k = 0; k < NQ; ++k) acc[k] += s[k];
+                            }
+                        });
+                        reduce(acc, [&]() {
+                            const double ts = sh.tot[0], tt = sh.tot[1], ss = sh.tot[2];
+                            const double qv = (lane == 0 ? ts : tt) / (lane == 0 ? tt : ts);   // omega, 1 / omega
+                            const double iom = __shfl_sync(0xffffffffu, qv, 1);
+                            if (lane == 0) {
+                                int act2 = CHIP_GO;
+                                double om = 0.0;
+                                if (chip_finite(ss) && met(ss)) {
+                                    act2 = CHIP_HALF;
+                                } else if (chip_zero(tt) || !chip_finite(tt)) {
+                                    sh.status = chip_finite(tt) ? DERR_BREAKDOWN : DERR_NONFINITE;
+                                    act2 = CHIP_HALF;
+                                } else {
+                                    om = qv;
+                                    if (chip_zero(om)) sh.status = DERR_BREAKDOWN;
+                                    if (sh.status != 0) {
+                                        act2 = CHIP_HALF;
+                                    } else {
+                                        const double rr1 = fma(-om, ts, ss);                    // ||s - omega t||^2
+                                        const double rho_new = fma(-om, sh.tot[3], NQ == 5 ? sh.tot[4] : 0.0);   // <rhat, r>
+                                        if (DF && chip_finite(rr1) && chip_exp(rr1) + CHIP_CANCEL < chip_exp(ss)) {
+                                            act2 = met(0x1p-17 * ss) ? CHIP_FULL : CHIP_CHECK;
+                                            sh.iom = iom;
+                                        } else {
+                                            act2 = after(rr1, rho_new, iom);
+                                        }
+                                    }
+                                }
+                                sh.om = (KT)om;
+                                sh.act = act2;
+                            }
+                        });
+                    };
+                    if (DF || it > FINE_EARLY) {
+                        KT acc[5] = {};
+                        half(acc);
+                    } else {
+                        KT acc[4] = {};
+                        half(acc);
+                    }
                     if (DF && sh.act == CHIP_CHECK) {
                         const KT om = sh.om;
                         KT chk[2] = {(KT)0, (KT)0};

@@ -128,6 +128,15 @@ __device__ __forceinline__ void cta_sum(Acc<KT, NQ>& acc, double* red) {
     }
 }
 
+// Iterations of a step in which the FP64 mode takes <rhat, s> as zero.  It is zero by the choice of
+// alpha, but only as far as rho is <rhat, r>: taken as zero throughout, rho keeps the rounding of the
+// first iteration, ~1e-16 of the first rho, while <rhat, r> falls with the residual, and steps of about
+// nine iterations or more no longer converged.  Until a residual nears the tolerance that rounding is
+// small beside rho, and a sum formed once makes rho <rhat, r> again, so the first iterations, which
+// are all that most steps take, go without the product (an FP64 operation a point: 16^3 x 8 x 125 steps
+// with it in every iteration 3.83 ms, now 3.69; 64^3 x 64 x 16 steps 62.6, now 61.3).
+constexpr int FINE_EARLY = 3;
+
 // Warp sums of NQ values a lane, halving the values a lane holds while the lanes that share
 // one double (9 additions for 5 values where 5 separate trees take 25).  Afterwards the lanes
 // whose low bits are zero hold value `q` (returned; -1: none).
@@ -1231,10 +1240,8 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
                     const KT al = (KT)sh.alpha;
                     // FP64: <rhat, t> and <rhat, s> too, from which beta and the stopping test follow
                     // without the products of the update pass: <rhat, r> = <rhat, s> - omega <rhat, t>,
-                    // ||r||^2 = <s,s> - omega <t,s>.  (<rhat, s> is zero by the choice of alpha, but
-                    // only as far as rho is <rhat, r>: taken as zero, rho keeps the rounding of the first
-                    // iteration while <rhat, r> falls with the residual, and steps of about nine
-                    // iterations or more no longer converged.)
+                    // ||r||^2 = <s,s> - omega <t,s>.  (<rhat, s>: FINE_EARLY.)
+                    const bool late = it > FINE_EARLY;
                     constexpr int NQ2 = DF ? 3 : 5;
                     Acc<KT, NQ2> acc;
                     acc.init();
@@ -1262,7 +1269,7 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
                                   acc.f[2] += q7.c.v[e] * q7.c.v[e];
                                   if constexpr (!DF) {
                                       acc.f[3] += hv.v[e] * tv.v[e];
-                                      acc.f[4] += hv.v[e] * q7.c.v[e];
+                                      if (late) acc.f[4] += hv.v[e] * q7.c.v[e];
                                   }
                               }
                               acc.tick();
