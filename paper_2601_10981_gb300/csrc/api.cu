@@ -1258,15 +1258,15 @@ pr_status pr_fine_sweep_batch(pr_ctx* const* ctxs, const int* ks, int count) {
                         "(with or without a stored perturbation)");
         if (!owner || c->groups_max > owner->groups_max) owner = c;
     }
-    FineArgs a{};
-    a.g = grid_of(owner);
-    a.njobs = count;
-    a.B = 0;
+    // steady and time-dependent flows run different kernels: one launch each, so that a context
+    // sweeps as it does alone
+    FineArgs args[2]{};
     for (int i = 0; i < count; ++i) {
         pr_ctx* c = ctxs[i];
         const int k = ks[i];
         const long long Ng = c->Ng;
-        FineJob& J = a.jobs[i];
+        FineArgs& a = args[c->tdep ? 1 : 0];
+        FineJob& J = a.jobs[a.njobs++];
         J.tab = c->tab;
         J.tdep = c->tdep ? 1 : 0;
         J.rk4 = c->o.fine == PR_FINE_RK4 ? 1 : 0;
@@ -1295,14 +1295,17 @@ pr_status pr_fine_sweep_batch(pr_ctx* const* ctxs, const int* ks, int count) {
         J.pert = c->pert ? (c->fp32 ? (const void*)c->pert32 : (const void*)c->pert) : nullptr;
         a.B += J.B;
     }
-    a.ws = owner->fws;
-    a.ust = owner->ust;
-    a.part = owner->fpart;
-    a.bar = owner->fbar;
-    a.bar_groups = owner->groups_max;
-    a.G = owner->o.group_ctas;
-    a.spin_limit = owner->o.spin_limit;
-    a.err = owner->derr;
+    for (FineArgs& a : args) {
+        a.g = grid_of(owner);
+        a.ws = owner->fws;
+        a.ust = owner->ust;
+        a.part = owner->fpart;
+        a.bar = owner->fbar;
+        a.bar_groups = owner->groups_max;
+        a.G = owner->o.group_ctas;
+        a.spin_limit = owner->o.spin_limit;
+        a.err = owner->derr;
+    }
     // order: each context's earlier work -> the launch on the owner's stream -> each
     // context's later work
     for (int i = 0; i < count; ++i) {
@@ -1313,8 +1316,11 @@ pr_status pr_fine_sweep_batch(pr_ctx* const* ctxs, const int* ks, int count) {
     }
     {
         pr_ctx* c = owner;
-        PR_CUDA(cudaMemsetAsync(c->fbar, 0, sizeof(unsigned) * 4 * c->groups_max, c->st));
-        PR_CUDA(launch_fine(a, c->fp32, c->o.ctas_per_sm, c->groups_max, c->st));
+        for (const FineArgs& a : args) {
+            if (a.njobs == 0) continue;
+            PR_CUDA(cudaMemsetAsync(c->fbar, 0, sizeof(unsigned) * 4 * c->groups_max, c->st));
+            PR_CUDA(launch_fine(a, c->fp32, c->o.ctas_per_sm, c->groups_max, c->st));
+        }
         PR_CUDA(cudaEventRecord(c->ev[7], c->st));
     }
     for (int i = 0; i < count; ++i) {

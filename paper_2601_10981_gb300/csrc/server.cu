@@ -59,12 +59,13 @@ struct Req {
     std::string err;
 };
 
-// n, box length, precision, fine integrator, stored perturbation (one launch runs one
-// stencil kind)
-using ShapeKey = std::tuple<int, double, int, int, int>;
+// n, box length, precision, fine integrator, stored perturbation, time-dependent flow (one launch
+// runs one stencil kind, and a tuned group size is that of one kernel)
+using ShapeKey = std::tuple<int, double, int, int, int, int>;
 
 ShapeKey shape_of(const pr_request& r) {
-    return ShapeKey(r.grid.n, r.grid.L, r.opts.precision, r.opts.fine, r.flow.pert ? 1 : 0);
+    const bool tdep = r.flow.kind == PR_FLOW_PAPER_KOLMOGOROV || r.flow.kind == PR_FLOW_PAPER_ABC;
+    return ShapeKey(r.grid.n, r.grid.L, r.opts.precision, r.opts.fine, r.flow.pert ? 1 : 0, tdep ? 1 : 0);
 }
 
 }  // namespace
