@@ -99,11 +99,16 @@ typedef struct pr_opts {
     double aug_tol;         /* no augmentation if ||d~|| <= aug_tol ||U||; default 1e-12  */
     int group_ctas;         /* CTAs cooperating on one subinterval in the fine sweep (its
                                tile-planes split evenly over them; capped at their count);
-                               0: every co-resident CTA slot over the subintervals.
-                               Small grids (n <= 48 FP32, 34 FP64) run in the shared memory of
-                               one thread-block cluster a subinterval: 0 chooses its size, a
-                               positive value sets it (at most 16; n <= 40 FP32, 28 FP64)    */
-    int ctas_per_sm;        /* resident CTAs per SM for the fine sweep; 0: occupancy max  */
+                               0: chosen by how many subintervals the sweep has.
+                               Steady flows on small grids (implicit Euler, n <= 48 FP32, 34
+                               FP64) run in the shared memory of one thread-block cluster a
+                               subinterval: 0 chooses its size, and whether that is the
+                               faster form.  A positive value is its size (at most 16): the
+                               nearest that fits for n <= 36 FP32, 28 FP64; on the larger of
+                               these grids a size that fits, any other the general kernels   */
+    int ctas_per_sm;        /* resident CTAs per SM of the fine sweep's streaming kernel; 0:
+                               occupancy max.  (FP32 steady flows on large grids run one CTA
+                               per SM after the first step, small grids whole clusters)      */
     long long spin_limit;   /* polls of an in-kernel barrier or mbarrier before
                                PR_ERR_TIMEOUT (default 1<<22, a few seconds; 0: one
                                non-blocking check, so a wait not already complete fails).
@@ -238,9 +243,9 @@ pr_status pr_coarse_sweep(pr_ctx* ctx, int k);
 pr_status pr_fine_sweep_batch(pr_ctx* const* ctxs, const int* ks, int count);
 
 /* Autotuner of the fine launch shape (no counterpart in the paper): times `steps` fine
- * steps of all n_sub subintervals from the current iterate for CTA-group sizes G = the
- * co-resident CTA count / n_sub and G = (n / tile rows) * 2^j up to the co-resident CTA
- * count, keeps the fastest in the
+ * steps of all n_sub subintervals from the current iterate for the CTA-group sizes that
+ * suit the kernels of this grid and flow (the cluster sizes, powers of two, whole multiples
+ * of a tile column, and the automatic choice's), keeps the fastest in the
  * context (pr_opts.group_ctas) and returns it (best_ms: its time, may be NULL).  Needs
  * iteration 0 done and no phase of the next iteration started; leaves the iterate
  * unchanged.  Synchronises. */

@@ -1337,17 +1337,13 @@ pr_status pr_tune_fine(pr_ctx* c, int steps, int* best_group_ctas, double* best_
     if (c->k_done < 0 || c->phase != 0 || !c->ws_ready)
         return fail(c, PR_ERR_STATE, "pr_tune_fine needs iteration 0 done and no phase in progress");
     steps = std::max(1, std::min(steps, c->S));
-    const int NY = c->n / fine_tile_rows(c->n);
-    const int maxc = fine_max_ctas(c->n, c->fp32, c->o.ctas_per_sm);
     const double* u_in = c->Ubuf[c->cur];
     const int B = c->N;
     double best = 1e300;
     int bestG = 0;
-    // candidates: the even split of every CTA slot over the subintervals, then whole
-    // multiples of the y-block columns
-    std::vector<int> cand{std::max(1, maxc / B)};
-    for (int z = 1; NY * z <= maxc && z <= c->n; z *= 2)
-        if (NY * z != cand[0]) cand.push_back(NY * z);
+    const bool implicit = c->o.fine == PR_FINE_IMPLICIT_EULER && !c->tdep;
+    const std::vector<int> cand =
+        fine_tune_groups(c->n, c->fp32, implicit, c->pert != nullptr, B, c->o.ctas_per_sm, c->o.spin_limit > 0);
     for (int Gc : cand) {
         c->o.group_ctas = Gc;
         float ms = 0.f;

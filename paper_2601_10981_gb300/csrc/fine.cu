@@ -410,6 +410,27 @@ static cudaError_t launch_streaming(FineArgs a, bool fp32, int mode, int ctas_pe
     return e;
 }
 
+// The kernel that a positive group size reaches depends on it (fine_chip_plan), so a size stands for
+// a kernel and its shape.
+std::vector<int> fine_tune_groups(int n, bool fp32, bool implicit, bool pert, int B, int ctas_per_sm, bool waits) {
+    std::vector<int> all, own;
+    const int sms = device_sms(), maxc = fine_max_ctas(n, fp32, ctas_per_sm);
+    if (implicit && waits) fine_chip_groups(n, fp32, B, &all);
+    if (implicit && waits && fp32 && !pert && fine_fused_takes(n)) {
+        fine_fused_groups(n, B, sms, &own);
+    } else {   // the even split of every CTA slot over the subintervals, whole multiples of the y-blocks
+        const int NY = n / fine_tile_rows(n);
+        own.push_back(std::max(1, maxc / B));
+        for (int z = 1; NY * z <= maxc && z <= n; z *= 2) own.push_back(NY * z);
+    }
+    ChipChoice ch;
+    for (int G : own)
+        if (!(implicit && waits && fine_chip_plan(n, fp32, B, G, &ch))) all.push_back(G);
+    std::sort(all.begin(), all.end());
+    all.erase(std::unique(all.begin(), all.end()), all.end());
+    return all;
+}
+
 cudaError_t launch_fine(FineArgs a, bool fp32, int ctas_per_sm, int max_groups, cudaStream_t st) {
     if (a.B <= 0) return cudaSuccess;
     const int n = a.g.n;
@@ -433,7 +454,10 @@ cudaError_t launch_fine(FineArgs a, bool fp32, int ctas_per_sm, int max_groups, 
         if (fine_chip_plan(n, fp32, a.B, a.G, &ch)) return launch_fine_chip(a, fp32, ch, max_groups, st);
     }
     // Large grids of the FP32 mode: fine_kernel for the first step, fused_kernel, and fine_kernel
-    // again for the items it leaves (usually none).  The group size is the caller's in each.
+    // again for the items it leaves (usually none).  A caller's group size is fused_kernel's, which
+    // runs one CTA an SM; fine_kernel takes as many times that as it has resident, while its CTAs keep
+    // eight tile-planes (40^3 x 4 x 40 steps in groups of 2: 2.99 -> 2.63 ms, 48^3 x 64 6.50 -> 5.61).  A
+    // single CTA waits for no other and stays single.
     // The second launch reads both u_0 and u_1, which u_out holds: not in place.
     bool in_place = false;
     for (int j = 0; j < a.njobs; ++j) {
@@ -449,10 +473,15 @@ cudaError_t launch_fine(FineArgs a, bool fp32, int ctas_per_sm, int max_groups, 
             first.jobs[j].S = 1;
             first.jobs[j].resume = nullptr;
         }
+        if (a.G > 1) {
+            const int occ = fine_max_ctas(n, fp32, ctas_per_sm) / device_sms();
+            first.G = std::max(a.G, std::min(a.G * occ, n / fine_tile_rows(n) * n / 8));
+        }
         cudaError_t e = launch_streaming(first, fp32, mode, ctas_per_sm, max_groups, st);
         if (e != cudaSuccess || most == 1) return e;
         e = launch_fine_fused(a, max_groups, st);
         if (e != cudaSuccess) return e;
+        a.G = first.G;
         return launch_streaming(a, fp32, mode, ctas_per_sm, max_groups, st);
     }
     for (int j = 0; j < a.njobs; ++j) a.jobs[j].resume = nullptr;

@@ -785,11 +785,12 @@ static int chip_clusters(int C) {
 // planes a CTA at most fit, so 11-CTA clusters in eight turns); FP32 16^3 x 16 1.27 -> 0.37
 // (fine_kernel), 32^3 x 64 2.4 -> 1.5, 40^3 x 8 1.23 -> 0.75, but 40^3 x 64 2.8 -> 3.4 and
 // 48^3 x 16 2.0 -> 2.3 (fused_kernel), 45^3 x 16 3.4 -> 2.5 (fine_kernel).
-// A caller who fixes group_ctas gets that C (the nearest that fits) on the grids where the
-// cluster always wins, whatever B, and fine_kernel beyond: the result of a subinterval then
-// does not depend on how many share the launch.
+// A caller who fixes group_ctas gets that C whatever B, so that the result of a subinterval does not
+// depend on how many share the launch: the nearest that fits on the grids where the cluster always
+// wins, and on larger ones the other kernels where no cluster of that size fits.
 bool fine_chip_plan(int n, bool fp32, int B, int group_ctas, ChipChoice* out) {
-    if (n < 4 || (group_ctas > 0 && n > (fp32 ? 36 : 28))) return false;
+    if (n < 4) return false;
+    const bool nearest = n <= (fp32 ? 36 : 28);
     double best = 0.0;
     out->C = 0;
     const double n2 = (double)n * n;
@@ -800,6 +801,7 @@ bool fine_chip_plan(int n, bool fp32, int B, int group_ctas, ChipChoice* out) {
         if (smem == 0) continue;
         double t;
         if (group_ctas > 0) {
+            if (!nearest && C != group_ctas) continue;
             t = std::abs(C - group_ctas);
         } else {
             const double npl = (n + C - 1) / C;
@@ -823,6 +825,16 @@ bool fine_chip_plan(int n, bool fp32, int B, int group_ctas, ChipChoice* out) {
     const double streamed = fp32 ? (n % 4 ? 45000.0 + 0.11 * pts : 50000.0 + 0.023 * pts)
                                  : 150000.0 + (n % 4 ? 0.95 : 0.55) * pts;
     return best < streamed;
+}
+
+void fine_chip_groups(int n, bool fp32, int B, std::vector<int>* out) {
+    ChipChoice ch;
+    if (fine_chip_plan(n, fp32, B, 0, &ch)) out->push_back(ch.C);
+    for (int C = 1, last = 0; C <= CHIP_MAXC; ++C) {   // the smallest cluster of each slab height
+        if (!fine_chip_plan(n, fp32, B, C, &ch) || ch.C != C || (n + C - 1) / C == last) continue;
+        last = (n + C - 1) / C;
+        out->push_back(C);
+    }
 }
 
 cudaError_t launch_fine_chip(const FineArgs& a, bool fp32, const ChipChoice& ch, int max_groups, cudaStream_t st) {

@@ -854,6 +854,30 @@ bool fine_fused_takes(int n) {
 // turns of the groups over the B items times the barriers and reductions (12,000 cycles) and the
 // planes of a CTA with the ones beyond its ends (2,700 each at 2048 points; 64^3 x 64, 40 steps:
 // G = 1 14.0, 2 7.2, 4 8.0, 9 9.5, 19 12 ms).
+static int fused_group(int planes, int B, int max_groups, int sms) {
+    double best = 0.0;
+    int G = 1;
+    for (int c = 1; c <= std::min(sms, planes); ++c) {
+        const int groups = std::min(std::min(B, max_groups), sms / c);
+        const double t = (double)((B + groups - 1) / groups) * (12000.0 + 2700.0 * ((planes + c - 1) / c + 3));
+        if (c == 1 || t < best) {
+            best = t;
+            G = c;
+        }
+    }
+    return G;
+}
+
+void fine_fused_groups(int n, int B, int sms, std::vector<int>* out) {
+    int TY, threads, slots;
+    size_t smem;
+    if (!fused_geom(n, &TY, &threads, &slots, &smem)) return;
+    const int planes = n / TY * n, most = std::min(sms, planes);
+    out->push_back(fused_group(planes, B, B, sms));
+    out->push_back(std::max(1, std::min(sms / std::max(1, B), most)));   // all groups at once
+    for (int c = 1; c <= most; c *= 2) out->push_back(c);
+}
+
 cudaError_t launch_fine_fused(FineArgs a, int max_groups, cudaStream_t st) {
     int threads;
     size_t smem;
@@ -867,17 +891,7 @@ cudaError_t launch_fine_fused(FineArgs a, int max_groups, cudaStream_t st) {
     a.NY = a.g.n / a.TY;
     const int planes = a.NY * a.g.n;
     int G = std::min(a.G, std::min(sms, planes));
-    if (G <= 0) {
-        double best = 0.0;
-        for (int c = 1; c <= std::min(sms, planes); ++c) {
-            const int groups = std::min(std::min(a.B, max_groups), sms / c);
-            const double t = (double)((a.B + groups - 1) / groups) * (12000.0 + 2700.0 * ((planes + c - 1) / c + 3));
-            if (G <= 0 || t < best) {
-                best = t;
-                G = c;
-            }
-        }
-    }
+    if (G <= 0) G = fused_group(planes, a.B, max_groups, sms);
     a.G = G;
     a.numGroups = std::min(std::min(a.B, max_groups), std::max(1, sms / G));
     void* args[] = {&a};

@@ -1599,6 +1599,7 @@ FineFn fine_fn_pert(bool fp32, int W, int KF, int KS);   // FINE_MODE_IMPLICIT_P
 // The FP32 mode's large grids in two passes a step (fine_fused.cu), steps 2 .. S after a launch of
 // the first one; whether the grid suits it.
 bool fine_fused_takes(int n);
+void fine_fused_groups(int n, int B, int sms, std::vector<int>* out);   // group sizes worth timing
 cudaError_t launch_fine_fused(FineArgs a, int max_groups, cudaStream_t st);
 
 // The same propagator on chip (fine_chip.cu): grids whose Krylov vectors fit the shared memory
@@ -1609,6 +1610,7 @@ struct ChipChoice {
     size_t smem;
 };
 bool fine_chip_plan(int n, bool fp32, int B, int group_ctas, ChipChoice* out);
+void fine_chip_groups(int n, bool fp32, int B, std::vector<int>* out);   // cluster sizes worth timing
 cudaError_t launch_fine_chip(const FineArgs& a, bool fp32, const ChipChoice& ch, int max_groups, cudaStream_t st);
 
 }  // namespace pr

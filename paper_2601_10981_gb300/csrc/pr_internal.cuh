@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "../../include/parareal.h"
 
 namespace pr {
@@ -222,6 +224,9 @@ cudaError_t launch_fine(FineArgs a, bool fp32, int ctas_per_sm, int max_groups,
                         cudaStream_t st);
 // Largest number of co-resident CTAs of the fine kernel for this grid size.
 int fine_max_ctas(int n, bool fp32, int ctas_per_sm);
+// Group sizes (pr_opts.group_ctas) worth timing for B subintervals, the automatic choice's among them;
+// waits: the context's waits may last (spin_limit > 0).
+std::vector<int> fine_tune_groups(int n, bool fp32, bool implicit, bool pert, int B, int ctas_per_sm, bool waits);
 size_t fine_part_doubles(int max_ctas);   // FineArgs::part
 int fine_tile_rows(int n);
 int fine_block_threads(int n);
