@@ -17,10 +17,10 @@
 // step adds the increment, forms the true residual by another setup (without the state's
 // update) and takes another iteration from there.
 // The first step, whose start is far from its solution, is fine_kernel's (a launch of one step
-// before this one; delta is u_1 - u_0), and so is the rest of an item that needs more than
-// FUSED_AGAIN further iterations (a launch after this one resumes it at the state before that
-// step).  The general iteration in this kernel would cost its registers (64^3 x 64, 40 steps:
-// 12.1 ms with it, its spills reloaded in the marches, 7.6 without).
+// before this one; delta is u_1 - u_0), and so is the rest of an item from a step on that needs more
+// than FUSED_MOST iterations (a launch after this one resumes it at the state before that step).
+// The general iteration in this kernel would cost its registers (64^3 x 64, 40 steps: 12.1 ms with
+// it, its spills reloaded in the marches, 7.6 without).
 //
 // What bounds it: latency and issue slots, not bytes (64^3 x 64: 4.4 TB/s of traffic, 41 % of
 // the issue slots).  A CTA (one an SM, 256 threads with two units of four points each, so that
@@ -49,7 +49,13 @@ constexpr int FUSED_RSLOTS = 6;   // planes of r in the krylov pass, three of th
 // floats, hold ~1e-6)
 constexpr double FUSED_CANCEL = 1e-4;
 constexpr long long FUSED_DRAIN = 1 << 20;   // tries of a wait for copies in flight before leaving
-constexpr int FUSED_AGAIN = 2;   // further iterations of an item's steps before it is left to fine_kernel
+// Iterations a step may take before its item is left to fine_kernel.  ms, fine_kernel alone and this
+// kernel, by iterations a step: 64^3 x 64 x 40 steps 2.0 22.2 and 13.3, 3.0 30.7 and 19.4; x 16 6.6 and
+// 4.5, 9.0 and 6.6; 96^3 x 16 x 40 2.0 41.5 and 14.0; 128^3 x 16 x 30 2.0 33.7 and 18.2.  From four on
+// the iterations here, each restarted from the true residual, lose to fine_kernel's and the item goes
+// back at its first such step, which then is done twice: x 30 steps 5.0 36.8 and 38.5, 8.7 59.9 and
+// 62.1; limits of 5 and 9 only make that step longer (38.8, 39.4).
+constexpr int FUSED_MOST = 3;
 
 struct FusedShared : FineShared {
     float wred[5 * 32];
@@ -313,7 +319,6 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
         bool hasx = true;             // delta holds an increment
         // the increment so far is delta + al r + om (ga r - al q)
         float al = 0.0f, om = 0.0f, ga = 0.0f;
-        int again = FUSED_AGAIN;
         xc = 0, xd = 7 * Ng, rc = Ng, rd = 2 * Ng;
         int left = 0;                 // the step that is left to fine_kernel
         // owned points, a tile plane at a time
@@ -774,7 +779,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
                     })) return;
                 ++it;
                 conv = sh.flag == 1;
-                if (sh.flag == 2 || (!conv && (it >= J.maxit || again-- == 0))) {
+                if (sh.flag == 2 || (!conv && it >= min(J.maxit, FUSED_MOST))) {
                     left = j;
                     --it;
                     break;
