@@ -453,10 +453,14 @@ def two_pass_bytes_per_dof_step(lin_iters: float, dM: int, has_f: bool) -> float
 
 
 def fine_two_pass(precision: str, w) -> bool:
-    """Whether the fine sweep of this workload takes the two-pass form (grids above the on-chip
-    form's)."""
-    return precision == "fp32" and w.n % 4 == 0 and w.n > 48 and w.flow.pert_seed == 0 and \
-        not w.flow.kind.startswith("paper_")
+    """Whether the fine sweep of this workload takes the two-pass form: steady unperturbed flows on
+    grids above the on-chip form's that a tile of rows divides (fused_geom in fine_fused.cu: 256
+    threads of four points each on every second row, eight rows and 96 threads or more)."""
+    if precision != "fp32" or w.n % 4 or w.n <= 48 or w.flow.pert_seed or w.flow.kind.startswith("paper_"):
+        return False
+    lanes = w.n // 4
+    ty = max((t for t in range(1, w.n + 1) if w.n % t == 0 and (t + 1) // 2 * lanes <= 256), default=0)
+    return ty >= 8 and (ty + 1) // 2 * lanes >= 96
 
 
 def serving_sample(n_req: int, rate: float, t_scale: float, seed: int = 5):
