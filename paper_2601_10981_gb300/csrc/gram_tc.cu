@@ -323,6 +323,9 @@ __device__ __forceinline__ int col_exp(unsigned long long m) {
     return m ? (int)((m >> 52) & 0x7FF) - 1023 + 3 : 0;
 }
 
+// a column that holds an infinity or a NaN: its digits mean nothing, its products are NaN
+__device__ __forceinline__ bool col_bad(unsigned long long m) { return m >= 0x7FF0000000000000ull; }
+
 // 2^sc * S, rounded once to the nearest double (ties to even)
 __device__ __forceinline__ double i128_to_double(__int128 S, int sc) {
     if (S == 0) return 0.0;
@@ -567,7 +570,8 @@ __global__ void __launch_bounds__(N2_THREADS, 1) gram_tc32_kernel(GramArgs a, lo
                     }
                     for (; cc < chunks; ++cc) S += src[(size_t)cc * cs];
                     const int sc = col_exp(colmax[(size_t)b * ld + i]) + col_exp(colmax[(size_t)b * ld + j]) - 84;
-                    const double g = i128_to_double(S, sc);
+                    const bool bad = col_bad(colmax[(size_t)b * ld + i]) || col_bad(colmax[(size_t)b * ld + j]);
+                    const double g = bad ? nan("") : i128_to_double(S, sc);
                     Gb[(size_t)i * a.ldG + j] = g;
                     Gb[(size_t)j * a.ldG + i] = g;
                 }
@@ -892,6 +896,7 @@ __global__ void __launch_bounds__(640, 1) gram_tc_kernel(GramArgs a, int CH, int
                     for (int e = 0; e < 8; ++e) sum += v[e];
                 }
                 for (; cc < chunks; ++cc) sum += src[(size_t)cc * outsz];
+                if (col_bad(colmax[(size_t)b * ld + i]) || col_bad(colmax[(size_t)b * ld + j])) sum = nan("");
                 Gb[(size_t)i * a.ldG + j] = sum;
                 Gb[(size_t)j * a.ldG + i] = sum;
             }
