@@ -751,7 +751,7 @@ static size_t chip_smem(int n, bool fp32, int C, int* keep) {
 }
 
 // Clusters of C CTAs that run at once with one CTA an SM (a GPC holds whole clusters only, so
-// large ones leave SMs idle), asked of the driver once per device.
+// large ones leave SMs idle), asked of the driver once per device; 0: none fits, or no answer.
 static int chip_clusters(int C) {
     static std::mutex mu;
     static std::vector<std::array<int, CHIP_MAXC + 1>> known;
@@ -770,9 +770,9 @@ static int chip_clusters(int C) {
         int m = 0;
         if (cudaOccupancyMaxActiveClusters(&m, fn, &cfg) != cudaSuccess) {
             cudaGetLastError();
-            m = 0;
+            return 0;
         }
-        have = std::max(1, m) + 1;
+        have = std::max(0, m) + 1;
     }
     return have - 1;
 }
@@ -800,15 +800,17 @@ bool fine_chip_plan(int n, bool fp32, int B, int group_ctas, ChipChoice* out) {
         const size_t smem = chip_smem(n, fp32, C, &keep);
         if (smem == 0) continue;
         double t;
+        if (group_ctas > 0 && !nearest && C != group_ctas) continue;
+        const int at_once = chip_clusters(C);
+        if (at_once == 0) continue;
         if (group_ctas > 0) {
-            if (!nearest && C != group_ctas) continue;
             t = std::abs(C - group_ctas);
         } else {
             const double npl = (n + C - 1) / C;
             const double fix = fp32 ? 12000.0 : 28000.0;
             const double work = fp32 ? (n % 4 ? 6.0 : 2.7) * n2 * (npl + 0.7) : 70.0 * n2 * npl;
             // clusters in turn, or two an SM where they fit: those share its pipes
-            const int at_once = chip_clusters(C), deep = (B + at_once - 1) / at_once;
+            const int deep = (B + at_once - 1) / at_once;
             if (smem > CHIP_SMEM / 2 || deep == 1) t = deep * (fix + work);
             else t = (deep / 2) * (fix + 2.0 * work) + (deep % 2) * (fix + work);
         }
