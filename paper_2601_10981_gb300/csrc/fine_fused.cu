@@ -316,7 +316,6 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
         const float dtf = (float)J.dt, c1 = (float)(J.dt * J.eps / (a.g.h * a.g.h));
         const float* ff = J.f32;
         double* snap_b = J.snap ? reinterpret_cast<double*>(J.snap) + (size_t)lb * J.n_snap * Ng : nullptr;
-        bool hasx = true;             // delta holds an increment
         // the increment so far is delta + al r + om (ga r - al q)
         float al = 0.0f, om = 0.0f, ga = 0.0f;
         xc = 0, xd = 7 * Ng, rc = Ng, rd = 2 * Ng;
@@ -409,13 +408,13 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
                         unsigned long long* mb = &sh.full[slot];
                         const bool fin = ff && zp >= zlo && zp < zhi;
                         if (warp == 0 && lane == 0) {
-                            const int planes = 2 + (hasx ? 1 : 0) + (upd ? 2 : 0);
+                            const int planes = 3 + (upd ? 2 : 0);
                             mbar_expect(mb, (unsigned)((planes * PL + (fin ? TY * n : 0)) * 4));
                         }
                         for (int w = warp; w < 6; w += nwarps) {
                             if (w == 5) {
                                 if (lane == 0 && fin) bulk_load(sl + 5 * PL, ff + zp * n2 + y0 * n, TY * n * 4, mb);
-                            } else if (lane < 3 && (w < 2 || (w == 2 ? hasx : upd))) {
+                            } else if (lane < 3 && (w < 3 || upd)) {
                                 int row, cnt, at;
                                 piece_of(lane, y0, 1, row, cnt, at);
                                 const float* base = w < 2 ? ust + uin + w * Ng : Wk + (w == 2 ? xc : (w == 3 ? rc : qo));
@@ -427,7 +426,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
                     auto operand = [&](const float* sl, int o, P4& hi, P4& lo, P4& d) -> P4 {
                         hi = ld4(sl + o);
                         lo = ld4(sl + PL + o);
-                        d = hasx ? ld4(sl + 2 * PL + o) : zero4();
+                        d = ld4(sl + 2 * PL + o);
                         if (upd) {
                             const P4 r = ld4(sl + 3 * PL + o);
                             const P4 sv = fma4s(nal2, ld4(sl + 4 * PL + o), mul4s(ga2, r));
@@ -563,9 +562,6 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
                         }
                         sh.flag = conv;
                         sh.rho = rr0;
-                        sh.alpha = 1.0;
-                        sh.omega = 1.0;
-                        sh.beta = 0.0;
                     })) return;
                 unsigned x = xc;
                 xc = xd;
@@ -574,7 +570,6 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
                 rc = rd;
                 rd = x;
             }
-            if (al != 0.0f) hasx = true;
             al = om = ga = 0.0f;
             bool conv = sh.flag != 0;
             // ================ krylov: q = (A - I) r and the products of r, q, (A - I) q
@@ -807,7 +802,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_kernel(const __grid_co
                 float hi[4], lo[4], d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
                 unpack4(ld4(ust + uo + i), hi);
                 unpack4(ld4(ust + uo + Ng + i), lo);
-                if (hasx && !left) unpack4(ld4(Wk + xc + i), d);
+                if (!left) unpack4(ld4(Wk + xc + i), d);
                 if (al != 0.0f && !left) {
                     float r4[4], q4[4];
                     unpack4(ld4(Wk + rc + i), r4);
