@@ -134,7 +134,7 @@ __device__ __forceinline__ void cta_sum(Acc<KT, NQ>& acc, double* red) {
 // nine iterations or more no longer converged.  Until a residual nears the tolerance that rounding is
 // small beside rho, and a sum formed once makes rho <rhat, r> again, so the first iterations, which
 // are all that most steps take, go without the product (an FP64 operation a point: 16^3 x 8 x 125 steps
-// with it in every iteration 3.83 ms, now 3.69; 64^3 x 64 x 16 steps 62.6, now 61.3).
+// with it in every iteration 3.83 ms, now 3.69; 64^3 x 64 x 16 steps 62.6, now 61.1).
 constexpr int FINE_EARLY = 3;
 
 // Warp sums of NQ values a lane, halving the values a lane holds while the lanes that share
@@ -1274,7 +1274,7 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
                               }
                               acc.tick();
                           });
-                    if (!finish(acc, [&](const double* s) {
+                    auto post = [&](const double* s) {
                     const double ts = s[0], tt2 = s[1], ss = s[2];
                     const int half = sqrt(ss) <= sh.thr;
                     if (!half) {
@@ -1289,7 +1289,7 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
                     sh.flag = half;
                     if constexpr (!DF) {   // 0: go on, 1: delta += alpha p only, 2: the step is done
                         if (!half && sh.status == 0) {
-                            const double rr1 = fma(-sh.omega, ts, ss), rho_new = fma(-sh.omega, s[3], s[4]);
+                            const double rr1 = fma(-sh.omega, ts, ss), rho_new = fma(-sh.omega, s[3], late ? s[4] : 0.0);
                             sh.flag = 2;
                             if (!isfinite(rr1)) sh.status = DERR_NONFINITE;
                             else if (sqrt(fmax(rr1, 0.0)) <= sh.thr) {}
@@ -1304,7 +1304,21 @@ __global__ void __launch_bounds__(256, 2) fine_kernel(FineArgs a) {
                             sh.flag = 1;
                         }
                     }
-                    })) return;
+                    };
+                    bool ok;
+                    if (DF || late) {
+                        ok = finish(acc, post);
+                    } else {
+                        Acc<KT, 4> four;
+                        four.init();
+#pragma unroll
+                        for (int q = 0; q < NQ2 - 1; ++q) {
+                            four.s[q] = acc.s[q];
+                            four.f[q] = acc.f[q];
+                        }
+                        ok = finish(four, post);
+                    }
+                    if (!ok) return;
                 }
                 if constexpr (!DF) {
                     // ---------------- ph3: delta += alpha p + omega s ; r = s - omega t if it goes on
