@@ -234,7 +234,8 @@ pr_status pr_coarse_sweep(pr_ctx* ctx, int k);
 /* pr_fine_sweep for several contexts at once (no counterpart in the paper: it serves
  * several problems on one GPU).  ks[i] is the iteration of ctxs[i]; all contexts need
  * the same n, box and precision, count <= 16, each context at most once.  Their
- * subintervals share one persistent launch of the fine kernel, one job per context,
+ * subintervals share one persistent launch of the fine kernel (steady and time-dependent
+ * flows one each: their kernels differ), one job per context,
  * issued on the stream of the context with the most CTA groups and ordered after each
  * context's earlier work and before its later work; each context then continues with
  * pr_pod_update.  With a fixed pr_opts.group_ctas the results are bit-identical to
@@ -406,7 +407,8 @@ pr_status pr_op_apply_L_noalloc(pr_ctx* ctx, const double* d_in, double* d_out, 
  * box and precision share persistent launches (pr_fine_sweep_batch, up to 16 requests
  * each), then each request's POD update and coarse sweep on its own stream, so that the
  * requests' work overlaps on the device.  A small request thus finishes while a large
- * one is mid-solve.  The fine CTA-group size is tuned once per (n, box, precision) by
+ * one is mid-solve.  The fine CTA-group size is tuned once per (n, box, precision, fine
+ * integrator, stored perturbation, time-dependent flow) by
  * pr_tune_fine on the first request admitted with opts.group_ctas = 0 and used for every
  * later request of that shape; a request with group_ctas > 0 keeps its own, and then
  * gives the same result alone and in a mix.

@@ -18,7 +18,7 @@
 //      POD update and coarse sweep on its own stream, then its event.
 // A small request therefore finishes while a large one is mid-solve, and its iterations
 // never wait for another request's.  The CTA-group size of the fine launch is tuned once
-// per (n, precision) by pr_tune_fine on the first request admitted with group_ctas = 0,
+// per shape (ShapeKey) by pr_tune_fine on the first request admitted with group_ctas = 0,
 // and reused for every later request of that shape, so that batched and single launches
 // tile a subinterval the same way (results are then identical alone and in the mix).
 #include "../../include/parareal.h"
