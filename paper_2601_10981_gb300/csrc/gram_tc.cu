@@ -689,7 +689,7 @@ __device__ __forceinline__ void add96(unsigned (&w)[3], long long H, long long L
 
 // 17 warps: five share one SM sub-partition's 16K registers, so at most 96 a thread (the bound of
 // 640 threads says so); the exact sums, touched once a window, live in shared memory
-__global__ void __launch_bounds__(640, 1) gram_tc_kernel(GramArgs a, int CH, int chunks,
+__global__ void __launch_bounds__(640, 1) gram_tc_kernel(GramArgs a, int CH, int chunks, int SH, int nsub,
                                                                 const unsigned long long* colmax, int ld,
                                                                 int* err, long long limit) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -731,7 +731,15 @@ __global__ void __launch_bounds__(640, 1) gram_tc_kernel(GramArgs a, int CH, int
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = s_tmem;
-    const int Ng = (int)a.Ng, units = a.B * chunks;
+    // An item's points are cut into chunks of CH, whose sums are rounded, and these into nsub units of
+    // SH points (fewer in the last chunk), whose sums stay exact where a chunk has several
+    const int Ng = (int)a.Ng;
+    const int upi = (chunks - 1) * nsub + (Ng - (chunks - 1) * CH + SH - 1) / SH, units = a.B * upi;
+    auto span = [&](int r, int& lo, int& hi) {   // unit r of an item
+        const int c = min(r / nsub, chunks - 1);
+        lo = c * CH + (r - c * nsub) * SH;
+        hi = min(min(Ng, (c + 1) * CH), lo + SH);
+    };
 
     if (warp == 16) {
         // ---------------- MMA issue (one thread) ----------------
@@ -739,7 +747,9 @@ __global__ void __launch_bounds__(640, 1) gram_tc_kernel(GramArgs a, int CH, int
             int gs = 0, gw = 0;
             bool bad = false;
             for (int u = blockIdx.x; u < units; u += gridDim.x) {
-                const int len = min(Ng - (u % chunks) * CH, CH);
+                int lo, hi;
+                span(u % upi, lo, hi);
+                const int len = hi - lo;
                 for (int rel = 0; rel < len; rel += TC_PTS, ++gs) {
                     const bool first = rel % TC_WIN == 0;
                     if (first && !bad && !mbar_wait_f(tempty, (gw & 1) ^ 1, &s_fail, limit)) bad = true;
@@ -787,9 +797,9 @@ __global__ void __launch_bounds__(640, 1) gram_tc_kernel(GramArgs a, int CH, int
     const double* c = nullptr;
     auto set_unit = [&]() {
         if (u >= units) return;
-        const int b = u / chunks;
-        lo = p0 = (u - b * chunks) * CH;
-        hi = min(Ng, lo + CH);
+        const int b = u / upi;
+        span(u - b * upi, lo, hi);
+        p0 = lo;
         c = col < a.KA[b] ? reinterpret_cast<const double*>(a.colsA[(size_t)b * a.ldcols + col]) : nullptr;
     };
     double x[8];
@@ -848,14 +858,20 @@ __global__ void __launch_bounds__(640, 1) gram_tc_kernel(GramArgs a, int CH, int
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         mbar_arrive(tempty);   // the tiles may be overwritten
         if (!plast) return;
-        // ---- the unit's partial: 2^7 top + bottom (64 rows, two warps on), rounded once
+        // ---- the unit's partial: 2^7 top + bottom (64 rows, two warps on); a chunk rounded once, or,
+        // of several units a chunk, the upper triangle in 128-bit integers, row by row
         tc_prod_sync();
-        const int b = pu / chunks, chunk = pu - b * chunks;
+        const int b = pu / upi, unit = pu - b * upi;
         const int K = a.KA[b];
-        const size_t outsz = (size_t)a.maxKA * a.maxKB;
-        double* mypart = a.part + ((size_t)b * chunks + chunk) * outsz;
+        const int mk = a.maxKA;
+        const size_t outsz = (size_t)mk * a.maxKB, tri = (size_t)mk * (mk + 1) / 2;
+        double* mypart = a.part + ((size_t)b * chunks + unit) * outsz;
+        __int128* bexact = reinterpret_cast<__int128*>(a.part) + (size_t)b * upi * tri;
+        auto at = [&](int i, int j) { return (size_t)(i * mk - i * (i - 1) / 2 + (j - i)); };
+        auto rounded = [&](__int128 S, int i, int j) {
+            return i128_to_double(S, col_exp(colmax[(size_t)b * ld + i]) + col_exp(colmax[(size_t)b * ld + j]) - 70);
+        };
         if (top && irow < K) {
-            const int ei = col_exp(colmax[(size_t)b * ld + irow]);
 #pragma unroll 1
             for (int j = 0; j < 16; ++j) {
                 const int jj = 16 * cq + j;
@@ -865,8 +881,9 @@ __global__ void __launch_bounds__(640, 1) gram_tc_kernel(GramArgs a, int CH, int
                     return ((__int128)(int)v[2 * TC_PROD + o] << 64) |
                            ((unsigned long long)v[TC_PROD + o] << 32 | v[o]);
                 };
-                mypart[(size_t)irow * a.maxKB + jj] =
-                    i128_to_double((word(0) << 7) + word(64), ei + col_exp(colmax[(size_t)b * ld + jj]) - 70);
+                const __int128 S = (word(0) << 7) + word(64);
+                if (nsub == 1) mypart[(size_t)irow * a.maxKB + jj] = rounded(S, irow, jj);
+                else bexact[unit * tri + at(irow, jj)] = S;
             }
         }
         // the last unit of item b sums the chunk partials in chunk order
@@ -874,7 +891,7 @@ __global__ void __launch_bounds__(640, 1) gram_tc_kernel(GramArgs a, int CH, int
         tc_prod_sync();
         if (tid == 0) {
             const unsigned ticket = atom_add_acq_rel_u32(a.counter + b, 1u);
-            s_last = (ticket == (unsigned)chunks - 1u);
+            s_last = (ticket == (unsigned)upi - 1u);
         }
         tc_prod_sync();
         if (s_last) {
@@ -888,6 +905,14 @@ __global__ void __launch_bounds__(640, 1) gram_tc_kernel(GramArgs a, int CH, int
                 const double* src = bpart + (size_t)i * a.maxKB + j;
                 double sum = 0.0;
                 int cc = 0;
+                if (nsub > 1) {   // the same chunk sums
+                    const __int128* se = bexact + at(i, j);
+                    for (int r = 0; cc < chunks; ++cc) {
+                        __int128 S = 0;
+                        for (const int r1 = min(upi, (cc + 1) * nsub); r < r1; ++r) S += se[r * tri];
+                        sum += rounded(S, i, j);
+                    }
+                }
                 for (; cc + 8 <= chunks; cc += 8) {
                     double v[8];
 #pragma unroll
@@ -912,7 +937,7 @@ __global__ void __launch_bounds__(640, 1) gram_tc_kernel(GramArgs a, int CH, int
         const int q = gs % TC_NS;
         const bool mine = c != nullptr;
         const int cu = u, rel = p0 - lo, len = hi - lo;   // the stage at hand
-        if (rel == 0) ce = col_exp(mine ? colmax[(size_t)(u / chunks) * ld + col] : 0ull) + 1020;
+        if (rel == 0) ce = col_exp(mine ? colmax[(size_t)(u / upi) * ld + col] : 0ull) + 1020;
         unsigned zl[8], zh[8];
         if (mine) {
 #pragma unroll
@@ -1006,18 +1031,25 @@ cudaError_t launch_gram_tc(const GramArgs& a, unsigned long long* colmax, int ld
         ++g_launch_count;
         return cudaGetLastError();
     }
-    // wide form, one CTA an SM (the tiles take all 512 tensor-memory columns).  It rounds a unit's
-    // sums, and an item's Gram may not depend on how many items share the call: units of the context's
-    // items.  (Exact 128-bit partials, rounded at the end, would allow any units, but Grams of windows
+    // wide form, one CTA an SM (the tiles take all 512 tensor-memory columns).  It rounds a chunk's
+    // sums, and an item's Gram may not depend on how many items share the call: chunks of the context's
+    // items.  (Exact sums over an item, rounded at the end, would allow any chunks, but Grams of windows
     // with fewer modes than columns, so rounded, take the Jacobi iteration more sweeps: four windows
     // of 64 on 128^3, 13.8 -> 15.4 ms a POD call.)
     const int cw = units(std::max(1, a.items));
     const int CHw = (int)(((a.Ng + cw - 1) / cw + TC_PTS - 1) / TC_PTS * TC_PTS);
     const int chunksw = (int)((a.Ng + CHw - 1) / CHw);
+    // A call of fewer items cuts the chunks into units that stay exact (one window of 54 on 64^3 in a
+    // context of 16: 0.97 -> 0.27 ms); their partials are K (K + 1) doubles where the other kernels'
+    // are K^2.
+    const int most = std::min(units(a.B), (int)((long long)chunks * a.maxKA / (a.maxKA + 1)));
+    const int want = std::max(1, most / chunksw);
+    const int SH = ((CHw + want - 1) / want + TC_PTS - 1) / TC_PTS * TC_PTS;
+    const int nsub = (CHw + SH - 1) / SH;
     e = cudaFuncSetAttribute((const void*)gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
     if (e != cudaSuccess) return e;
-    const int grid = std::max(1, std::min(sms, a.B * chunksw));
-    gram_tc_kernel<<<grid, TC_THREADS, TC_SMEM, st>>>(a, CHw, chunksw, colmax, ld, err, spin_limit);
+    const int grid = std::max(1, std::min(sms, a.B * chunksw * nsub));
+    gram_tc_kernel<<<grid, TC_THREADS, TC_SMEM, st>>>(a, CHw, chunksw, SH, nsub, colmax, ld, err, spin_limit);
     ++g_launch_count;
     return cudaGetLastError();
 }

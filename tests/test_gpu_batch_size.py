@@ -46,7 +46,8 @@ def test_double_float_gram_in_clusters(gpu, n, K, B):
 
 
 # the wide form over units of one item to several: a single unit, ragged ones, 33 columns to 64
-@pytest.mark.parametrize("n,K,B", [(9, 64, 3), (45, 64, 6), (64, 40, 5), (72, 33, 4)])
+@pytest.mark.parametrize("n,K,B", [(9, 64, 3), (45, 64, 6), (64, 40, 5), (72, 33, 4), (37, 50, 12),
+                                   (64, 54, 16)])
 def test_tensor_gram(gpu, n, K, B):
     bd, torch = gpu
     w = pi.Workload("gram", n, pi.Flow("abc"), 0.05, 1.0, B, 1e-3, n_snap=64, m_cap=32)
